@@ -121,7 +121,9 @@ typedef struct {
                       step's two Krylov steps, likewise delta                   */
   int32_t profile; /* nonzero: launch kernels one by one (no CUDA graph) with
                       a CUDA event pair around every launch on the launching
-                      stream, and report per-kind device time below           */
+                      stream, and report per-kind device time below; a sector
+                      small enough to run whole steps in one kernel reports
+                      the time and number of that kernel's phases instead     */
   double* kernel_ms;        /* [ED_KERNEL_KINDS] summed event time per kind  */
   int64_t* kernel_launches; /* [ED_KERNEL_KINDS] launches per kind           */
 } ed_observables;
@@ -413,6 +415,10 @@ ed_status ed_set_workspace_limit(ed_ctx* ctx, int64_t bytes);
  * asynchronously and does not read the status).  No copy is left in flight
  * when a block ends.  withhold_copy = -1 (the default) turns the hook off.
  * ED_ERR_ARG for withhold_copy < -1 or wait_polls outside 0..2^32-1.
+ * Propagations that run whole steps in one kernel (small sectors, no pinned
+ * configuration) wait in grid-wide sums with the same poll limit; for them
+ * withhold_copy >= 0 makes one thread block leave out its contribution to
+ * that sum (counted from 0 per launch), with the same result.
  * (No passage of the paper: a check of the library's own failure path.)    */
 ed_status ed_set_wait_fault(int withhold_copy, int64_t wait_polls);
 

@@ -42,7 +42,7 @@ size_t Engine::device_bytes() const {
          d_emap_.bytes +
          d_partials_.bytes + d_counters_.bytes + d_coefs_.bytes + d_coefs_obs_.bytes +
          d_V_.bytes + d_w_.bytes + d_out_.bytes + d_owned_x1_.bytes + d_maps_.bytes +
-         d_map_off_.bytes + d_map_spin_.bytes + d_ovl_.bytes + d_psiT_.bytes;
+         d_slots_.bytes + d_map_off_.bytes + d_map_spin_.bytes + d_ovl_.bytes + d_psiT_.bytes;
 }
 
 static std::atomic<int> g_forced_cfg{-1};
@@ -401,6 +401,32 @@ std::string Engine::setup(const EngineConfig& cfg, const std::vector<SectorDev>&
   args_.col_map = static_cast<const ApplyBlock*>(d_cmap_.p);
   args_.n_col_blocks = (int)cmap.size();
   args_.partials = static_cast<double*>(d_partials_.p);
+  return setup_persistent(nv == 1 && !cfg.overlaps && !up_tabs.empty() ? up_tabs[vecs_[0].sector]
+                                                                       : nullptr,
+                          vec_ok);
+}
+
+std::string Engine::setup_persistent(const SpinTable* up, bool vec_ok) {
+  kry_grid_ = 0;
+  if (!up) return "";
+  const SectorDev& sd = sectors_[vecs_[0].sector];
+  int dev = 0, sms = 0, coop = 0;
+  ED_TRY(cudaGetDevice(&dev));
+  ED_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  ED_TRY(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  const int grid = std::min(std::min(sms, kKrylovMaxGrid), sd.dim_up);
+  if (!coop || grid < 1) return "";
+  kry_rows_ = (sd.dim_up + grid - 1) / grid;
+  kry_deg_ = 1;
+  for (int r = 0; r < up->dim; ++r) kry_deg_ = std::max(kry_deg_, up->off[r + 1] - up->off[r]);
+  kry_vec_ = vec_ok;
+  kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_, cfg_.fp64);
+  if (kry_smem_ > 227 * 1024) return "";
+  int ctas = 0;
+  ED_TRY(krylov_prepare(cfg_.fp64, kry_vec_, kry_smem_, &ctas));
+  if (ctas < 1) return "";
+  ED_TRY(d_slots_.alloc(kKrylovSlotBytes));
+  kry_grid_ = grid;
   return "";
 }
 
@@ -556,6 +582,40 @@ std::string Engine::capture(cudaStream_t s) {
 std::string Engine::run(int n_steps, bool profile, double* kernel_ms, int64_t* launches,
                         cudaStream_t s) {
   const bool f = cfg_.fp64;
+  // Sectors whose rows fit the chip's shared memory run whole sub-steps in
+  // the persistent kernel, kKrylovSteps of them per launch (a launch of the
+  // largest such sector then lasts a few tens of ms).  A pinned
+  // configuration asks for the separate kernels.  In profile mode the kernel
+  // itself adds up the time of its phases.
+  constexpr int kKrylovSteps = 16;
+  if (kry_grid_ > 0 && forced_apply_config() < 0) {
+    KrylovArgs k;
+    k.a = args_;
+    k.slots = static_cast<ulonglong2*>(d_slots_.p);
+    k.rows = kry_rows_;
+    k.max_deg = kry_deg_;
+    k.energy = cfg_.energy ? 1 : 0;
+    DevMem prof;
+    if (profile) {
+      ED_TRY(prof.alloc(2 * KK_COUNT * sizeof(uint64_t)));
+      ED_TRY(cudaMemsetAsync(prof.p, 0, prof.bytes, s));
+    }
+    k.prof = static_cast<uint64_t*>(prof.p);
+    for (int n = 0; n == 0 || n < n_steps; n += kKrylovSteps) {
+      k.n_steps = std::min(kKrylovSteps, n_steps - n);
+      ED_TRY(launch_krylov(f, kry_vec_, k, kry_grid_, kry_smem_, s));
+    }
+    if (profile) {
+      uint64_t h[2 * KK_COUNT];
+      ED_TRY(cudaMemcpyAsync(h, prof.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+      ED_TRY(cudaStreamSynchronize(s));
+      for (int i = 0; i < KK_COUNT; ++i) {
+        if (kernel_ms) kernel_ms[i] = 1e-6 * (double)h[2 * i];
+        if (launches) launches[i] = (int64_t)h[2 * i + 1];
+      }
+    }
+    return "";
+  }
   // observables at t_0 (also sets beta0 and the first scale)
   ED_TRY(launch_observe(f, args_, n_ew_, s));
   if (have_overlaps_) {

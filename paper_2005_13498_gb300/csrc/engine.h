@@ -117,6 +117,9 @@ class Engine {
   std::string launch_step(cudaStream_t s, bool profile, cudaEvent_t* ev, int* kind_of,
                           int* nev);
   std::string capture(cudaStream_t s);
+  // Whether the persistent Krylov kernel can run this engine's vector; sets
+  // its launch shape.
+  std::string setup_persistent(const SpinTable* up, bool vec_ok);
   // psi^T for the overlaps of vectors stored transposed (map mode 2)
   cudaError_t launch_psiT(cudaStream_t s);
 
@@ -139,6 +142,11 @@ class Engine {
   DevMem d_coefs_, d_coefs_obs_, d_V_, d_w_, d_out_, d_owned_x1_;
   DevMem d_maps_, d_map_off_, d_map_spin_, d_ovl_, d_psiT_;
   bool need_psiT_ = false;
+  // persistent Krylov kernel: grid 0 = not used
+  int kry_grid_ = 0, kry_rows_ = 0, kry_deg_ = 0;
+  bool kry_vec_ = false;
+  size_t kry_smem_ = 0;
+  DevMem d_slots_;
   cudaGraph_t graph_ = nullptr;
   cudaGraphExec_t exec_ = nullptr;
 };

@@ -190,6 +190,26 @@ cudaError_t launch_permute_cols_copy(bool fp64, const void* src, void* dst, int 
 cudaError_t launch_transpose(bool fp64, const void* in, void* out, int rows, int cols,
                              cudaStream_t s);
 
+// ---- persistent Krylov kernel (krylov.cu): n_steps sub-steps of vector 0 in
+// one cooperative launch
+constexpr int kKrylovMaxGrid = 160;   // CTAs (one per SM) of a launch
+constexpr size_t kKrylovSlotBytes = 4 * (size_t)kKrylovMaxGrid * sizeof(ulonglong2);
+struct KrylovArgs {
+  BatchArgs a;
+  ulonglong2* slots;   // [2 epochs][2 values][kKrylovMaxGrid] published partial sums (zeroed per launch)
+  int rows;          // most rows a CTA owns
+  int max_deg;       // most T_up entries of a row
+  int n_steps;       // sub-steps of this launch
+  int energy;        // record E(t) with a.coefs_obs
+  uint64_t* prof;    // null, or [KK_COUNT][2]: ns and number of each kind's phases
+};
+// Dynamic shared memory of a launch, and the CTAs per SM it allows (0: does
+// not fit); krylov_prepare raises the kernel's limit.
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, bool fp64);
+cudaError_t krylov_prepare(bool fp64, bool vec, size_t smem, int* ctas_per_sm);
+cudaError_t launch_krylov(bool fp64, bool vec, const KrylovArgs& k, int grid, size_t smem,
+                          cudaStream_t s);
+
 // ---- ground-state helpers (float64 only) ---------------------------------
 // partial[blk][i] = sum over block chunk of conj(V_i) w, i < k  (k <= 256)
 cudaError_t launch_multidot(const double2* V, int64_t ldV, int k,

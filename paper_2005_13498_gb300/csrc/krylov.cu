@@ -1,0 +1,974 @@
+// Persistent Krylov kernel: whole midpoint (or CFET4) sub-steps of one vector
+// in one cooperative launch, for sectors whose rows fit the shared memory of
+// the chip.
+//
+// With one kernel per Lanczos pass a small sector pays a launch, a chain of
+// dependent table loads, a tail and a cold start 2 m + 2 times per sub-step.
+// Here every CTA (one per SM) owns the rows c, c + G, c + 2 G, .. (G CTAs) for
+// the whole launch: they stay in shared memory as the tile the within-row
+// gathers (T_dn) read, w never leaves the CTA, the connection lists and the
+// ELL words stay in shared memory and L1, and per Lanczos step only two
+// grid-wide sums are left (alpha_j, then beta_j together with the visibility
+// of x_{j+1}, whose rows the T_up gathers of the other CTAs read through L2).
+// Measured per call, separate kernels -> this kernel: 20 steps of the 8-site
+// ring with energies (D = 4,900, m = 12, complex128) 7.67 -> 4.43 ms, 10 steps
+// of the 12-site torus (D = 853,776, m = 20, complex64) 8.40 -> 7.47 ms, two
+// CFET4 steps of it with energies in complex128 21.8 -> 15.1 ms.
+// What bounds it: for the ring the latency of the passes (4 us) and of the
+// sums (4.5 us each: 2.1 us from a CTA's store to the last CTA's successful
+// poll across the two dies, the rest dependent float64 additions at about
+// 50 ns); for the torus the shared-memory and L2 gathers (complex64, 21 of 37
+// us per Lanczos step) and the FP64 pipe (complex128, 183 us).
+// It is used when two copies of a CTA's rows fit its shared memory: up to
+// about 15 MB of state (D = 1.9 M in complex64, 0.95 M in complex128).
+//
+// Grid-wide sums: each CTA publishes its float64 partial as two 64-bit words
+// that carry the sum's epoch in their upper halves, and one warp of every CTA
+// polls all CTAs' words and adds them in CTA order, so that no counter, no
+// second round trip and no broadcast is needed and every CTA holds the same
+// total.  All scalars of the recursion (and the small exponential) are then
+// computed by every CTA alike.  Every poll is bounded: a wait that runs out
+// records ED_ERR_TIMEOUT and ends the CTA.  The launch is cooperative, so the
+// CTAs are resident together.
+#include "device.cuh"
+
+namespace ed {
+
+namespace {
+
+constexpr int kErrTimeout = 4;    // ED_ERR_TIMEOUT
+constexpr int kErrNumeric = 7;    // ED_ERR_NUMERIC
+constexpr int kUpBatch = 6;
+constexpr int kPollLanes = (kKrylovMaxGrid + 31) / 32;
+
+// complex64: two rows per 16-byte tile column, 20 warps at 96 registers;
+// complex128 (FP64-pipe bound): one row, 16 warps at 128 registers
+template <typename R> struct KCfg;
+template <> struct KCfg<float> { static constexpr int NT = 640, NR = 2; };
+template <> struct KCfg<double> { static constexpr int NT = 512, NR = 1; };
+
+// Scalars of the Lanczos recursion in shared memory, 1-based as LanczosState.
+struct Scalars {
+  double alpha[kMaxKrylov + 2], beta[kMaxKrylov + 2], inv[kMaxKrylov + 2];
+  double al[64], be[64], yre[64], yim[64], pre[64], pim[64];
+  double yprev_re[kMaxKrylov], yprev_im[kMaxKrylov];
+  double tot[2], part[2][4];
+  double beta0, scale, as, conv_delta;
+  double utab[kMaxSites + 1];   // U n
+  int m_eff, stop, status, conv, err, step;
+};
+
+// A published partial: the halves of a float64, each with the sum's epoch in
+// the upper 32 bits of its word, so that no ordering between the two words
+// is needed.  Slots of one sum lie side by side (16 bytes a CTA): a warp
+// polls 32 CTAs with four lines.
+__device__ __forceinline__ void ld_slot(const ulonglong2* p, uint64_t& w0, uint64_t& w1) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(w0), "=l"(w1) : "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_slot(ulonglong2* p, double v, uint32_t epoch) {
+  const uint64_t bits = (uint64_t)__double_as_longlong(v), e = (uint64_t)epoch << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(e | (bits >> 32)),
+               "l"(e | (bits & 0xffffffffull))
+               : "memory");
+}
+
+// v = sum over all CTAs of the threads' v (K values), left in S.tot of every
+// CTA; `after` runs in thread 0 with the totals in place, before the other
+// threads go on.  DATA: vectors written before the call are read by other
+// CTAs after it.  False when a wait gave up (in all threads of the CTA).
+template <int K, bool DATA, int NT, typename F>
+__device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Scalars& S,
+                                         const KrylovArgs& k, uint32_t& epoch, F&& after) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned full = 0xffffffffu;
+  constexpr int QW = 4;   // warps (one per SM sub-partition) that add the threads' values
+  double part[K];
+#pragma unroll
+  for (int kk = 0; kk < K; ++kk) {
+    if (kk > 0) __syncthreads();
+    redS[tid] = v[kk];
+    __syncthreads();
+    if (warp < QW) {
+      double s = 0.0;
+#pragma unroll
+      for (int i = 0; i < NT / (32 * QW); ++i) s += redS[tid + i * 32 * QW];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
+      part[kk] = s;
+    }
+  }
+  if (warp < QW && lane == 0)
+#pragma unroll
+    for (int kk = 0; kk < K; ++kk) S.part[kk][warp] = part[kk];
+  __syncwarp();
+  __syncthreads();
+  ++epoch;
+  if (warp == 0) {
+    const int G = gridDim.x;
+    ulonglong2* base = k.slots + (size_t)(epoch & 1u) * 2 * kKrylovMaxGrid;
+    if (lane == 0) {
+      if constexpr (DATA) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      const bool withheld = k.a.tma_withhold >= 0 && blockIdx.x == 0 &&
+                            epoch == (uint32_t)k.a.tma_withhold + 1u;   // test hook
+      if (!withheld)
+#pragma unroll
+        for (int kk = 0; kk < K; ++kk)
+          st_slot(base + kk * kKrylovMaxGrid + blockIdx.x,
+                  (S.part[kk][0] + S.part[kk][1]) + (S.part[kk][2] + S.part[kk][3]), epoch);
+    }
+    __syncwarp();
+    uint64_t w[kPollLanes][K][2];
+    bool all = false;
+    for (uint32_t it = 0; it < k.a.wait_limit && !all; ++it) {
+      all = true;
+#pragma unroll
+      for (int q = 0; q < kPollLanes; ++q)
+        if (lane + 32 * q < G)
+#pragma unroll
+          for (int kk = 0; kk < K; ++kk)
+            ld_slot(base + kk * kKrylovMaxGrid + lane + 32 * q, w[q][kk][0], w[q][kk][1]);
+#pragma unroll
+      for (int q = 0; q < kPollLanes; ++q)
+        if (lane + 32 * q < G)
+#pragma unroll
+          for (int kk = 0; kk < K; ++kk)
+            all = all && (uint32_t)(w[q][kk][0] >> 32) == epoch && (uint32_t)(w[q][kk][1] >> 32) == epoch;
+    }
+    const bool ok = __all_sync(full, all);
+    if constexpr (DATA) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+    if (ok) {
+#pragma unroll
+      for (int kk = 0; kk < K; ++kk) {
+        double s = 0.0;
+#pragma unroll
+        for (int q = 0; q < kPollLanes; ++q)
+          if (lane + 32 * q < G)
+            s += __longlong_as_double((long long)((w[q][kk][0] << 32) |
+                                                  (w[q][kk][1] & 0xffffffffull)));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(full, s, o);
+        if (lane == 0) S.tot[kk] = s;
+      }
+      if (lane == 0) after();
+    } else if (lane == 0) {
+      S.err = 1;
+    }
+  }
+  __syncwarp();
+  __syncthreads();
+  return !S.err;
+}
+
+// L2 loads of the column pair (2p, 2p+1) of a row: the vectors are written by
+// other SMs during the kernel, so nothing may come from L1.  SELF: the pair
+// may have been written by this thread since the last call of a function that
+// is not inlined; such loads are volatile and stay behind those stores.
+template <typename T4>
+__device__ __forceinline__ T4 ldl2(const T4* p) {
+  static_assert(sizeof(T4) == 16 || sizeof(T4) == 8, "16- or 8-byte loads");
+  T4 v;
+  if constexpr (sizeof(T4) == 16) {
+    uint64_t a, b;
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+    reinterpret_cast<uint64_t*>(&v)[0] = a;
+    reinterpret_cast<uint64_t*>(&v)[1] = b;
+  } else {
+    uint64_t a;
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+    *reinterpret_cast<uint64_t*>(&v) = a;
+  }
+  return v;
+}
+template <typename C, bool VEC, bool SELF>
+__device__ __forceinline__ void ldcg_pair(const C* row, int p, int dim, C& v0, C& v1) {
+  if constexpr (VEC) {
+    const float4* a = reinterpret_cast<const float4*>(row) + p;
+    const float4 f = SELF ? ldl2(a) : __ldcg(a);
+    v0.x = f.x; v0.y = f.y; v1.x = f.z; v1.y = f.w;
+  } else {
+    v0 = SELF ? ldl2(row + 2 * p) : __ldcg(row + 2 * p);
+    v1 = czero<C>();
+    if (2 * p + 1 < dim) v1 = SELF ? ldl2(row + 2 * p + 1) : __ldcg(row + 2 * p + 1);
+  }
+}
+
+template <typename C>
+__device__ __forceinline__ bool same(C a, C b) { return a.x == b.x && a.y == b.y; }
+
+// The off-diagonal part of H x for one item, NR tile rows x 64 columns (two
+// columns per lane): acc[r][h] of row r and column 2 p + h.
+//  complex64: T_dn over the ELL slots of the tile (two slots per turn, words
+//  two turns ahead), then T_up row by row with the signed coefficients,
+//  eight source rows in flight.
+__device__ __forceinline__ void off_diagonal(
+    const SectorDev& sd, const float2* tile, int t, int p, int pcl, int npairs, const float2* x,
+    const uint2* const (&list)[2], const int (&deg)[2], const float2* coefS, const float2* coefQ,
+    bool vec, bool, bool, float2 (&acc)[2][2]) {
+  constexpr int NR = 2;
+  using TIO = TileIO<float2, NR>;
+  const int lane = threadIdx.x & 31;
+  const int dim_dn = sd.dim_dn;
+  const int q0 = __ldg(sd.dn_tslot_off + t), q1 = __ldg(sd.dn_tslot_off + t + 1);
+  const uint32_t* ellp = TIO::ellp_for(sd.dn_ellp32, sd.dn_ellpr) + lane;
+  const uint2* grp2 = reinterpret_cast<const uint2*>(sd.dn_slot_grp);
+  float2 s0[NR], s1[NR];
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    s0[r] = s1[r] = make_float2(0.f, 0.f);
+    acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
+  }
+  auto flush = [&](uint32_t g) {
+    const float2 c = coefS[g];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      cmac(acc[r][0], c, s0[r]);
+      cmac(acc[r][1], c, s1[r]);
+      s0[r] = s1[r] = make_float2(0.f, 0.f);
+    }
+  };
+  // Odd warps take T_up first: the L2 round trips of one half of the warps
+  // overlap the shared-memory gathers of the other.
+#pragma unroll 1
+  for (int ph = 0; ph < 2; ++ph) {
+    if (ph == 0) {
+      if (q0 >= q1) continue;
+      uint32_t na = __ldg(ellp + (size_t)q0 * 32), nb = __ldg(ellp + (size_t)(q0 + 1) * 32);
+      uint2 ng = __ldg(grp2 + (q0 >> 1));
+      uint32_t gcur = ng.x;
+      for (int q = q0; q < q1; q += 2) {
+        const uint32_t ea = na, eb = nb;
+        const uint2 gg = ng;
+        if (q + 2 < q1) {
+          na = __ldg(ellp + (size_t)(q + 2) * 32);
+          nb = __ldg(ellp + (size_t)(q + 3) * 32);
+          ng = __ldg(grp2 + ((q + 2) >> 1));
+        }
+        uint32_t oa0, oa1, ob0, ob1;
+        float ga0, ga1, gb0, gb1;
+        TIO::unpack<float>(ea, oa0, oa1, ga0, ga1);
+        TIO::unpack<float>(eb, ob0, ob1, gb0, gb1);
+        float2 a0[NR], a1[NR], b0[NR], b1[NR];
+        TIO::load_off(tile, oa0, a0);
+        TIO::load_off(tile, oa1, a1);
+        TIO::load_off(tile, ob0, b0);
+        TIO::load_off(tile, ob1, b1);
+        if (gg.x != gcur) { flush(gcur); gcur = gg.x; }   // uniform over the warp
+#pragma unroll
+        for (int r = 0; r < NR; ++r) { cax(s0[r], ga0, a0[r]); cax(s1[r], ga1, a1[r]); }
+        if (gg.y != gcur) { flush(gcur); gcur = gg.y; }
+#pragma unroll
+        for (int r = 0; r < NR; ++r) { cax(s0[r], gb0, b0[r]); cax(s1[r], gb1, b1[r]); }
+      }
+      flush(gcur);
+    } else {
+      constexpr int NB = kUpBatch;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        float2 sa[2], sb[2];
+        sa[0] = sa[1] = sb[0] = sb[1] = make_float2(0.f, 0.f);
+        for (int e = 0; e < deg[r]; e += NB) {
+          float2 v[NB][2];
+          uint32_t cs[NB];
+#pragma unroll
+          for (int i = 0; i < NB; ++i)
+            if (e + i < deg[r]) {   // uniform over the warp
+              const uint2 en = list[r][e + i];
+              cs[i] = en.y;
+              const float2* src = x + en.x;
+              if (vec) ldcg_pair<float2, true, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
+              else ldcg_pair<float2, false, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
+            }
+#pragma unroll
+          for (int i = 0; i < NB; ++i)
+            if (e + i < deg[r]) {
+              const float2 c = coefQ[cs[i]];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                sa[h] = ffma2(make_float2(c.x, c.x), v[i][h], sa[h]);
+                sb[h] = ffma2(make_float2(c.y, c.y), v[i][h], sb[h]);
+              }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          acc[r][h].x += sa[h].x - sb[h].y;
+          acc[r][h].y += sa[h].y + sb[h].x;
+        }
+      }
+    }
+  }
+}
+
+//  complex128: FP64-pipe bound (a warp instruction occupies it for 16 cycles
+//  of the SM), so the operations count: T_dn slots and T_up entries of one
+//  bond group share one signed sum, a group whose coefficient equals the
+//  previous one's joins its sum, and a real coefficient costs half a complex
+//  product.  Per element of the 12-site torus that is 75 operations where
+//  separate sums with a product per group and direction take 104.  lo, hi:
+//  which of the lane's two columns the item covers (uniform over the warp).
+__device__ __forceinline__ void off_diagonal(
+    const SectorDev& sd, const double2* tile, int t, int p, int pcl, int npairs, const double2* x,
+    const uint2* const (&list)[1], const int (&deg)[1], const double2* coefS, const float2*,
+    bool, bool lo, bool hi, double2 (&acc)[1][2]) {
+  using C = double2;
+  using TIO = TileIO<C, 1>;
+  const int lane = threadIdx.x & 31;
+  const int dim_dn = sd.dim_dn;
+  const uint32_t* ellp = TIO::ellp_for(sd.dn_ellp32, sd.dn_ellpr) + lane;
+  const uint2* lst = list[0];
+  const int ne = deg[0];
+  int q = __ldg(sd.dn_tslot_off + t), e = 0;
+  const int q1 = __ldg(sd.dn_tslot_off + t + 1);
+  constexpr uint32_t kEnd = 0xFFFFu;
+  uint32_t word = 0u, gq = kEnd;
+  if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
+  uint32_t ge = e < ne ? lst[e].y & 0xFFu : kEnd;
+  C s0 = czero<C>(), s1 = s0, cur = s0;
+  acc[0][0] = acc[0][1] = s0;
+  auto flush = [&]() {
+    if (cur.y == 0.0) {   // uniform over the block
+      if (lo) { acc[0][0].x += cur.x * s0.x; acc[0][0].y += cur.x * s0.y; }
+      if (hi) { acc[0][1].x += cur.x * s1.x; acc[0][1].y += cur.x * s1.y; }
+    } else {
+      if (lo) cmac(acc[0][0], cur, s0);
+      if (hi) cmac(acc[0][1], cur, s1);
+    }
+  };
+  bool any = false;
+  for (;;) {
+    const uint32_t g = min(gq, ge);   // uniform over the warp
+    if (g == kEnd) break;
+    const C c = coefS[g];
+    if (!any) {
+      cur = c;
+      any = true;
+    } else if (!same(c, cur)) {
+      flush();
+      s0 = s1 = czero<C>();
+      cur = c;
+    }
+    // the group's first T_up rows load while its T_dn slots are gathered
+    constexpr int NB = 4;
+    C v[NB][2];
+    double sg[NB];
+    int nb = 0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      if (nb == i && e + i < ne) {
+        const uint2 m = lst[e + i];
+        if ((m.y & 0xFFu) == g) {
+          ldcg_pair<C, false, false>(x + m.x, pcl, dim_dn, v[i][0], v[i][1]);
+          sg[i] = (m.y >> 31) ? -1.0 : 1.0;
+          nb = i + 1;
+        }
+      }
+    }
+    while (gq == g) {
+      const uint32_t w = word;
+      ++q;
+      if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
+      else gq = kEnd;
+      uint32_t o0, o1;
+      double g0, g1;
+      TIO::unpack<double>(w, o0, o1, g0, g1);
+      C a0[1], a1[1];
+      TIO::load_off(tile, o0, a0);
+      TIO::load_off(tile, o1, a1);
+      if (lo) cax(s0, g0, a0[0]);
+      if (hi) cax(s1, g1, a1[0]);
+    }
+#pragma unroll
+    for (int i = 0; i < NB; ++i)
+      if (i < nb) {
+        if (lo) cax(s0, sg[i], v[i][0]);
+        if (hi) cax(s1, sg[i], v[i][1]);
+      }
+    e += nb;
+    while (e < ne && (lst[e].y & 0xFFu) == g) {
+      C u0, u1;
+      ldcg_pair<C, false, false>(x + lst[e].x, pcl, dim_dn, u0, u1);
+      const double s = (lst[e].y >> 31) ? -1.0 : 1.0;
+      if (lo) cax(s0, s, u0);
+      if (hi) cax(s1, s, u1);
+      ++e;
+    }
+    ge = e < ne ? lst[e].y & 0xFFu : kEnd;
+  }
+  if (any) flush();
+}
+
+// The a-posteriori check of step j (as k_conv_check), by one warp.
+__device__ __noinline__ void conv_check(Scalars& S, int j, double tau, double eps_tol) {
+  const int lane = threadIdx.x & 31;
+  for (int i = lane; i < 64; i += 32) {
+    S.al[i] = i < j ? S.alpha[i + 1] : 0.0;
+    S.be[i] = i < j - 1 ? S.beta[i + 1] : 0.0;
+  }
+  __syncwarp();
+  tridiag_expm_e1(S.al, S.be, j, tau, S.yre, S.yim);
+  double dn = 0.0, yn = 0.0;
+  for (int i = lane; i < j; i += 32) {
+    const double pr = i < j - 1 ? S.yprev_re[i] : 0.0, pi = i < j - 1 ? S.yprev_im[i] : 0.0;
+    dn += (S.yre[i] - pr) * (S.yre[i] - pr) + (S.yim[i] - pi) * (S.yim[i] - pi);
+    yn += S.yre[i] * S.yre[i] + S.yim[i] * S.yim[i];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    dn += __shfl_xor_sync(0xffffffffu, dn, o);
+    yn += __shfl_xor_sync(0xffffffffu, yn, o);
+  }
+  __syncwarp();
+  for (int i = lane; i < j; i += 32) {
+    S.yprev_re[i] = S.yre[i];
+    S.yprev_im[i] = S.yim[i];
+  }
+  if (lane == 0) {
+    const double ny = sqrt(yn);
+    const double delta = sqrt(dn) / ny;
+    const double eps = delta < 1.0 ? fmin(1.0 + ny, delta / (1.0 - delta) * ny) : 1.0 + ny;
+    // S.as holds the breakdown scale seen by step j until this pass' alpha
+    if (eps < eps_tol || S.beta[j] < eps_tol * S.as) {
+      S.conv_delta = delta;
+      S.conv = j;
+    }
+  }
+  __syncwarp();
+}
+
+// Dynamic shared memory: Scalars, Share, then the arrays of Share.  Every
+// function takes its pointers from here, so that the compiler knows them to
+// be shared memory (through a generic pointer the gathers of apply_pass ran
+// 1.5 x slower).
+extern __shared__ __align__(16) unsigned char smem_raw[];
+
+// The CTA's share of the sector: held in registers through the whole kernel
+// these would spill.
+struct Share {
+  SectorDev sd;
+  VecDev vd;
+  int off_w, off_q, off_c, off_l, off_d;   // byte offsets of the arrays below
+  int max_deg, nloc, ld, npairs, ntile, items, nwork;
+};
+constexpr int kOffShare = (sizeof(Scalars) + 15) & ~15;
+constexpr int kOffX = (kOffShare + sizeof(Share) + 15) & ~15;
+__device__ __forceinline__ Scalars& scalars() { return *reinterpret_cast<Scalars*>(smem_raw); }
+__device__ __forceinline__ Share& share() { return *reinterpret_cast<Share*>(smem_raw + kOffShare); }
+// rows of x_j and w: [tile rows][dim_dn + zero columns][NR]
+template <typename C> __device__ __forceinline__ C* tile_x() { return reinterpret_cast<C*>(smem_raw + kOffX); }
+template <typename C> __device__ __forceinline__ C* tile_w() { return reinterpret_cast<C*>(smem_raw + share().off_w); }
+// complex64: signed coefficients [1 + 2 n_groups]; coefficients [n_groups]
+__device__ __forceinline__ float2* coef_q() { return reinterpret_cast<float2*>(smem_raw + share().off_q); }
+template <typename C> __device__ __forceinline__ C* coef_s() { return reinterpret_cast<C*>(smem_raw + share().off_c); }
+// T_up entries [rows][max_deg]: source offset, slot or group; their numbers
+__device__ __forceinline__ uint2* up_list() { return reinterpret_cast<uint2*>(smem_raw + share().off_l); }
+__device__ __forceinline__ int* up_deg() { return reinterpret_cast<int*>(smem_raw + share().off_d); }
+
+// w = s_in H x - s_prev x_prev of the CTA's rows into tileW; returns the
+// thread's Re<x, w>.  (One function for the Lanczos and the energy passes:
+// inlined in each place it took the registers of both.)
+template <typename R, bool VEC>
+__device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
+                                          const typename C2T<R>::T* xp, R s_in, R s_prev) {
+  const Scalars& S = scalars();
+  const Share& h = share();
+  // the loads below must not move up across the grid-wide sum before the
+  // pass: they depend on pointers that are opaque from here on
+  asm volatile("" : "+l"(x) : : "memory");
+  asm volatile("" : "+l"(xp) : : "memory");
+  using C = typename C2T<R>::T;
+  constexpr int NR = KCfg<R>::NR;
+  using TIO = TileIO<C, NR>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int G = gridDim.x, cta = blockIdx.x;
+  const SectorDev& sd = h.sd;
+  const int dim_dn = sd.dim_dn, npairs = h.npairs, ntile = h.ntile, nloc = h.nloc;
+  const int pitch = h.ld * NR;
+  const C* const tileX = tile_x<C>();
+  C* const tileW = tile_w<C>();
+  const uint2* const list = up_list();
+  const int* const degS = up_deg();
+  const C* const coefS = coef_s<C>();
+  const float2* const coefQ = coef_q();
+  double dot = 0.0;
+  if (warp >= h.nwork) return dot;
+  // complex128 with warps to spare: an item per column of the lanes' pairs
+  // (a float64 instruction holds its SM sub-partition for 64 cycles, so one
+  // warp's chain is what a small sector waits for; 8-site ring: see k_krylov)
+  const int split = NR == 1 && 2 * h.items <= h.nwork ? 2 : 1;
+  for (int is = warp; is < h.items * split; is += h.nwork) {
+    const int it = split == 2 ? is >> 1 : is;
+    const bool lo = split == 1 || !(is & 1), hi = split == 1 || (is & 1);
+    const int b = it / ntile, t = it - b * ntile, p = 32 * t + lane;
+    const C* tile = tileX + b * pitch;
+    const uint2* lst[NR];
+    int deg[NR], urow[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int li = b * NR + r;
+      const bool have = li < nloc;
+      lst[r] = list + (have ? li : 0) * h.max_deg;
+      deg[r] = have ? degS[li] : 0;
+      urow[r] = cta + (have ? li : 0) * G;
+    }
+    C acc[NR][2];
+    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefS, coefQ, VEC, lo, hi, acc);
+    if (p >= npairs) continue;
+    const int d0 = 2 * p;
+    const bool has1 = hi && d0 + 1 < dim_dn;
+    const uint32_t dw0 = __ldg(sd.dn_word + d0), dw1 = has1 ? __ldg(sd.dn_word + d0 + 1) : 0u;
+    C xa[NR], xb[NR], oa[NR], ob[NR];
+    TIO::load(tile, d0, xa);
+    TIO::load(tile, d0 + 1, xb);
+    R da = (R)0;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      oa[r] = ob[r] = czero<C>();
+      if (b * NR + r >= nloc) continue;
+      const uint32_t uw = __ldg(sd.up_word + urow[r]);
+      R g0 = (R)S.utab[__popc(uw & dw0)], g1 = (R)S.utab[__popc(uw & dw1)];
+      if (sd.up_eps) {
+        const R eu = (R)__ldg(sd.up_eps + urow[r]);
+        g0 += eu + (R)__ldg(sd.dn_eps + d0);
+        g1 += eu + (has1 ? (R)__ldg(sd.dn_eps + d0 + 1) : (R)0);
+      }
+      C a0 = acc[r][0], a1 = acc[r][1];
+      a0.x += g0 * xa[r].x;
+      a0.y += g0 * xa[r].y;
+      a1.x += g1 * xb[r].x;
+      a1.y += g1 * xb[r].y;
+      C o0, o1;
+      if (xp) {
+        C p0, p1;
+        ldcg_pair<C, VEC, false>(xp + (size_t)urow[r] * dim_dn, p, dim_dn, p0, p1);
+        o0.x = s_in * a0.x - s_prev * p0.x;
+        o0.y = s_in * a0.y - s_prev * p0.y;
+        o1.x = s_in * a1.x - s_prev * p1.x;
+        o1.y = s_in * a1.y - s_prev * p1.y;
+      } else {
+        o0.x = s_in * a0.x; o0.y = s_in * a0.y;
+        o1.x = s_in * a1.x; o1.y = s_in * a1.y;
+      }
+      oa[r] = o0;
+      ob[r] = o1;
+      if (lo) da += xa[r].x * o0.x + xa[r].y * o0.y;
+      if (has1) da += xb[r].x * o1.x + xb[r].y * o1.y;
+    }
+    if (lo) TIO::store(tileW + b * pitch, d0, oa);
+    if (has1) TIO::store(tileW + b * pitch, d0 + 1, ob);
+    dot += (double)da;
+  }
+  return dot;
+}
+
+template <typename R, bool VEC>
+__global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
+  using C = typename C2T<R>::T;
+  constexpr int NT = KCfg<R>::NT, NR = KCfg<R>::NR, NW = NT / 32;
+  using TIO = TileIO<C, NR>;
+  Scalars& S = scalars();
+  Share& h = share();
+  __shared__ double redS[NT];
+  __shared__ C cf[kMaxKrylov + 1];
+  __shared__ C cf_lo;
+
+  const BatchArgs& a = k.a;
+  if (threadIdx.x == 0) {
+    h.vd = a.vec[0];
+    h.sd = a.sec[a.vec[0].sector];
+  }
+  __syncthreads();
+  const SectorDev& sd = h.sd;
+  const VecDev& vd = h.vd;
+  LanczosState* st = a.st;
+  const int dim_up = sd.dim_up, dim_dn = sd.dim_dn;
+  const int npairs = (dim_dn + 1) >> 1, ntile = (dim_dn + 63) >> 6;
+  const int G = gridDim.x, cta = blockIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nloc = (dim_up - cta + G - 1) / G;   // rows cta, cta + G, ..
+  const int nblk = (nloc + NR - 1) / NR;         // tile rows of NR rows
+  const int ld = dim_dn + kZeroCols;
+  const int RB = (k.rows + NR - 1) / NR;
+  const int tile_bytes = RB * ld * 16;
+  const int off_q = kOffX + 2 * tile_bytes;
+  const int off_c = off_q + (sizeof(R) == 4 ? (1 + 2 * a.n_groups) * 8 : 0);
+  const int off_l = off_c + a.n_groups * (int)sizeof(C);
+  C* const tileX = tile_x<C>();
+  C* const tileW = reinterpret_cast<C*>(smem_raw + kOffX + tile_bytes);
+  float2* const coefQ = reinterpret_cast<float2*>(smem_raw + off_q);
+  C* const coefS = reinterpret_cast<C*>(smem_raw + off_c);
+  uint2* const list = reinterpret_cast<uint2*>(smem_raw + off_l);
+  int* const degS = reinterpret_cast<int*>(list + (size_t)k.rows * k.max_deg);
+  C* x1 = static_cast<C*>(vd.x1);
+  C* V = static_cast<C*>(vd.V);
+  const int m = st->m;
+  const double eps_tol = st->eps_tol;
+  const int items = nblk * ntile;
+  // with the adaptive exit the last warp runs the checks beside the passes
+  const int nwork = eps_tol > 0.0 ? NW - 1 : NW;
+
+  // ---- once per launch: connection lists and rows of the CTA
+  for (int li = 0; li < nloc; ++li) {
+    const int u = cta + li * G;
+    const int e0 = __ldg(sd.up_off + u), ne = __ldg(sd.up_off + u + 1) - e0;
+    for (int i = tid; i < ne; i += NT) {
+      const uint32_t en = __ldg(sd.up_ent + e0 + i);
+      const uint32_t g = (en >> kEntGroupShift) & 0xFFu;
+      list[(size_t)li * k.max_deg + i] =
+          make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
+                     sizeof(R) == 4 ? 1u + 2u * g + (en >> 31) : g | (en & kEntSignBit));
+    }
+    if (tid == 0) degS[li] = ne;
+  }
+  for (int i = tid; i < RB * ld; i += NT) {
+    const int b = i / ld, d = i - b * ld;
+    C v[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int li = b * NR + r;
+      v[r] = li < nloc && d < dim_dn ? ldl2(x1 + (size_t)(cta + li * G) * dim_dn + d) : czero<C>();
+    }
+    TIO::store(tileX + (size_t)b * ld * NR, d, v);
+    C z[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) z[r] = czero<C>();
+    TIO::store(tileW + (size_t)b * ld * NR, d, z);
+  }
+  if (tid == 0) {
+    h.off_w = kOffX + tile_bytes;
+    h.off_q = off_q;
+    h.off_c = off_c;
+    h.off_l = off_l;
+    h.off_d = off_l + k.rows * k.max_deg * (int)sizeof(uint2);
+    h.max_deg = k.max_deg;
+    h.nloc = nloc;
+    h.ld = ld;
+    h.npairs = npairs;
+    h.ntile = ntile;
+    h.items = items;
+    h.nwork = nwork;
+    S.err = 0;
+    S.status = 0;
+    S.step = st->step;
+  }
+  for (int i = tid; i <= kMaxSites; i += NT) S.utab[i] = a.U * (double)i;
+  __syncthreads();
+  uint32_t epoch = 0;
+  const int step0 = S.step;
+
+  auto load_coefs = [&](const void* base, int step) {
+    const C* c = reinterpret_cast<const C*>(base) + (size_t)step * a.n_groups;
+    for (int g = tid; g < a.n_groups; g += NT) coefS[g] = c[g];
+    if constexpr (sizeof(R) == 4)
+      for (int i = tid; i <= 2 * a.n_groups; i += NT) {
+        float2 q = make_float2(0.f, 0.f);
+        if (i > 0) {
+          const float2 cc = reinterpret_cast<const float2*>(c)[(i - 1) >> 1];
+          const float sg = ((i - 1) & 1) ? -1.f : 1.f;
+          q = make_float2(sg * cc.x, sg * cc.y);
+        }
+        coefQ[i] = q;
+      }
+    // reconverge first: a few lanes of warp 0 wrote the coefficients, and
+    // without this the other warps were seen to read the previous ones right
+    // after the block barrier
+    __syncwarp();
+    __syncthreads();
+  };
+  // one pass over the items: f(tile row, column tile, column pair)
+  auto for_items = [&](auto&& f) {
+    for (int it = warp; it < items; it += nwork) {
+      if (warp >= nwork) break;
+      const int b = it / ntile, t = it - b * ntile;
+      f(b, t, 32 * t + lane);
+    }
+  };
+  // psi -> per-thread |psi|^2 and sum of double occupancies of tile values
+  auto weigh = [&](int b, int p, const C (&va)[NR], const C (&vb)[NR], double& n2, double& dd) {
+    const int d0 = 2 * p;
+    const bool has1 = d0 + 1 < dim_dn;
+    const uint32_t dw0 = __ldg(sd.dn_word + d0), dw1 = has1 ? __ldg(sd.dn_word + d0 + 1) : 0u;
+    R nl = (R)0, wl = (R)0;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (b * NR + r >= nloc) continue;
+      const uint32_t uw = __ldg(sd.up_word + cta + (b * NR + r) * G);
+      const R qa = va[r].x * va[r].x + va[r].y * va[r].y;
+      const R qb = has1 ? vb[r].x * vb[r].x + vb[r].y * vb[r].y : (R)0;
+      nl += qa + qb;
+      wl += (R)__popc(uw & dw0) * qa + (R)__popc(uw & dw1) * qb;
+    }
+    n2 += (double)nl;
+    dd += (double)wl;
+  };
+  // outputs and scalars of a state with |psi|^2 = tot[0], in thread 0
+  auto new_state = [&](int slot) {
+    const double n2 = S.tot[0];
+    const double b0 = sqrt(n2);
+    S.beta0 = b0;
+    S.inv[1] = b0 > 0.0 ? 1.0 / b0 : 0.0;
+    S.scale = 1.0;
+    S.m_eff = m;
+    S.conv = 0;
+    S.stop = b0 > 0.0 && isfinite(b0) ? 0 : 1;
+    if (!isfinite(b0)) S.status = kErrNumeric;
+    if (cta == 0) {
+      if (vd.out_docc) vd.out_docc[slot] = S.tot[1] / a.Ns;
+      if (vd.out_norm2) vd.out_norm2[slot] = n2;
+    }
+  };
+  auto energy = [&](int slot) -> bool {
+    load_coefs(a.coefs_obs, slot);
+    const double v[1] = {apply_pass<R, VEC>(x1, nullptr, (R)1, (R)0)};
+    return grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
+      if (cta == 0 && vd.out_energy) vd.out_energy[slot] = S.tot[0] / a.Ns;
+    });
+  };
+  // profile mode: time of the phase that ends here, by kernel kind (CTA 0)
+  uint64_t last = 0;
+  auto mark = [&](int kind) {
+    if (k.prof && cta == 0 && tid == 0) {
+      uint64_t now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (kind >= 0) {
+        k.prof[2 * kind] += now - last;
+        k.prof[2 * kind + 1] += 1;
+      }
+      last = now;
+    }
+  };
+  auto finish = [&]() {
+    if (tid == 0 && S.err) st->status = kErrTimeout;
+    if (tid == 0 && cta == 0 && !S.err) {
+      if (S.status) st->status = S.status;
+      st->step = S.step;
+      st->m_eff = S.m_eff;
+    }
+  };
+
+  // ---- observables of the state at the launch's first time
+  {
+    double v[2] = {0.0, 0.0};
+    for_items([&](int b, int t, int p) {
+      if (p >= npairs) return;
+      C xa[NR], xb[NR];
+      TIO::load(tileX + (size_t)b * ld * NR, 2 * p, xa);
+      TIO::load(tileX + (size_t)b * ld * NR, 2 * p + 1, xb);
+      weigh(b, p, xa, xb, v[0], v[1]);
+    });
+    if (!grid_sum<2, true, NT>(v, redS, S, k, epoch, [&]() { new_state(step0); })) { finish(); return; }
+    if (k.energy && step0 == 0 && !energy(0)) { finish(); return; }
+  }
+
+  for (int s = 0; s < k.n_steps; ++s) {
+    mark(-1);
+    load_coefs(a.coefs, S.step);
+    // ---- Lanczos recursion
+    for (int j = 1; j <= m && !S.stop; ++j) {
+      const C* x = j == 1 ? x1 : V + (size_t)(j - 2) * vd.D;
+      const C* xp = j < 2 ? nullptr : j == 2 ? x1 : V + (size_t)(j - 3) * vd.D;
+      const R s_in = (R)S.inv[j];
+      const R s_prev = j >= 2 ? (R)(S.beta[j - 1] * S.inv[j - 1]) : (R)0;
+      if (warp >= nwork && j >= 2) conv_check(S, j - 1, a.tau, eps_tol);
+      const double v[1] = {apply_pass<R, VEC>(x, xp, s_in, s_prev)};
+      if (!grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
+            const double re = S.tot[0];
+            S.alpha[j] = re * S.inv[j];
+            S.as = S.alpha[j] * S.inv[j];
+            if (!isfinite(re)) {
+              S.status = kErrNumeric;
+              S.stop = 1;
+              S.m_eff = j > 1 ? j - 1 : 1;
+            } else if (S.conv > 0) {
+              S.stop = 1;
+              S.m_eff = S.conv;
+            }
+          })) { finish(); return; }
+      mark(KK_APPLY);
+      if (S.stop || j == m) break;
+      // x_{j+1} = w - alpha_j s_j x_j, into the tile and V
+      const R as = (R)S.as;
+      C* xn = V + (size_t)(j - 1) * vd.D;
+      double nrm[1] = {0.0};
+      for_items([&](int b, int t, int p) {
+        if (p >= npairs) return;
+        const int d0 = 2 * p;
+        const bool has1 = d0 + 1 < dim_dn;
+        C* tx = tileX + (size_t)b * ld * NR;
+        C xa[NR], xb[NR], wa[NR], wb[NR];
+        TIO::load(tx, d0, xa);
+        TIO::load(tx, d0 + 1, xb);
+        TIO::load(tileW + (size_t)b * ld * NR, d0, wa);
+        TIO::load(tileW + (size_t)b * ld * NR, d0 + 1, wb);
+        R nl = (R)0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          C o0, o1;
+          o0.x = wa[r].x - as * xa[r].x;
+          o0.y = wa[r].y - as * xa[r].y;
+          o1.x = has1 ? wb[r].x - as * xb[r].x : (R)0;
+          o1.y = has1 ? wb[r].y - as * xb[r].y : (R)0;
+          xa[r] = o0;
+          xb[r] = o1;
+          if (b * NR + r < nloc) {
+            store_pair<C, VEC>(xn + (size_t)(cta + (b * NR + r) * G) * dim_dn, p, dim_dn, o0, o1);
+            nl += o0.x * o0.x + o0.y * o0.y + o1.x * o1.x + o1.y * o1.y;
+          }
+        }
+        TIO::store(tx, d0, xa);
+        if (has1) TIO::store(tx, d0 + 1, xb);
+        nrm[0] += (double)nl;
+      });
+      if (!grid_sum<1, true, NT>(nrm, redS, S, k, epoch, [&]() {
+            const double beta = sqrt(S.tot[0]);
+            const double sc = fmax(S.scale, fabs(S.alpha[j]));
+            S.beta[j] = beta;
+            S.as = sc;   // read by the check of step j
+            if (!isfinite(beta)) {
+              S.status = kErrNumeric;
+              S.stop = 1;
+              S.m_eff = j;
+            } else if (beta <= a.break_tol * sc) {
+              S.stop = 1;
+              S.m_eff = j;
+            } else {
+              S.inv[j + 1] = 1.0 / beta;
+              S.scale = fmax(sc, beta);
+            }
+          })) { finish(); return; }
+      mark(KK_UPDATE);
+    }
+    // ---- the small exponential (by every CTA alike)
+    const int n = S.m_eff;
+    const bool zero = !(S.beta0 > 0.0 && isfinite(S.beta0));
+    if (S.conv > 0 && S.conv == n && !zero) {   // y^(n) and delta are the check's
+      for (int i = tid; i < n; i += NT) { S.yre[i] = S.yprev_re[i]; S.yim[i] = S.yprev_im[i]; }
+      __syncthreads();
+    } else {
+      for (int i = tid; i < 64; i += NT) {
+        S.al[i] = i < n && !zero ? S.alpha[i + 1] : 0.0;
+        S.be[i] = i < n - 1 && !zero ? S.beta[i + 1] : 0.0;
+      }
+      __syncthreads();
+      if (warp == 0) tridiag_expm_e1(S.al, S.be, n, a.tau, S.yre, S.yim);
+      else if (warp == 1 && n > 1)
+        tridiag_expm_e1(S.al, S.be, n - 1, a.tau, S.pre, S.pim);
+      __syncthreads();
+      if (warp == 1) {
+        double dn = 0.0, yn = 0.0;
+        if (n > 1)
+          for (int i = lane; i < n; i += 32) {
+            const double pr = i < n - 1 ? S.pre[i] : 0.0, pi = i < n - 1 ? S.pim[i] : 0.0;
+            dn += (S.yre[i] - pr) * (S.yre[i] - pr) + (S.yim[i] - pi) * (S.yim[i] - pi);
+            yn += S.yre[i] * S.yre[i] + S.yim[i] * S.yim[i];
+          }
+        for (int o = 16; o > 0; o >>= 1) {
+          dn += __shfl_xor_sync(0xffffffffu, dn, o);
+          yn += __shfl_xor_sync(0xffffffffu, yn, o);
+        }
+        if (lane == 0) S.conv_delta = n > 1 ? sqrt(dn / yn) : 0.0;
+      }
+    }
+    if (warp == 0)
+      for (int i = lane; i < n; i += 32) {
+        const double f = zero ? 0.0 : S.beta0 * S.inv[i + 1];
+        const double re = f * S.yre[i], im = f * S.yim[i];
+        cf[i].x = (R)re;
+        cf[i].y = (R)im;
+        if (i == 0) {
+          cf_lo.x = (R)(re - (double)(R)re);
+          cf_lo.y = (R)(im - (double)(R)im);
+        }
+      }
+    __syncthreads();
+    if (tid == 0 && cta == 0) {
+      if (vd.out_delta) vd.out_delta[S.step] = S.conv_delta;
+      if (vd.out_meff) vd.out_meff[S.step] = n;
+    }
+    mark(KK_EXPM);
+    // ---- psi = sum_j c_j x_j (the order of k_combine), observables fused
+    double v[2] = {0.0, 0.0};
+    const int nv = zero ? 1 : n;
+    for_items([&](int b, int t, int p) {
+      if (p >= npairs) return;
+      const int d0 = 2 * p;
+      const bool has1 = d0 + 1 < dim_dn;
+      C pa[NR], pb[NR];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        pa[r] = pb[r] = czero<C>();
+        if (b * NR + r >= nloc) continue;
+        const size_t off = (size_t)(cta + (b * NR + r) * G) * dim_dn;
+        C x0, x1v;
+        ldcg_pair<C, VEC, true>(x1 + off, p, dim_dn, x0, x1v);
+        C o0 = czero<C>(), o1 = czero<C>();
+        cmac(o0, cf_lo, x0);
+        cmac(o1, cf_lo, x1v);
+        const C* Vr = V + off;
+#pragma unroll 8
+        for (int jj = 1; jj < nv; ++jj) {
+          C y0, y1;
+          ldcg_pair<C, VEC, true>(Vr + (size_t)(jj - 1) * vd.D, p, dim_dn, y0, y1);
+          cmac(o0, cf[jj], y0);
+          cmac(o1, cf[jj], y1);
+        }
+        cmac(o0, cf[0], x0);
+        cmac(o1, cf[0], x1v);
+        store_pair<C, VEC>(x1 + off, p, dim_dn, o0, o1);
+        pa[r] = o0;
+        pb[r] = o1;
+      }
+      TIO::store(tileX + (size_t)b * ld * NR, d0, pa);
+      if (has1) TIO::store(tileX + (size_t)b * ld * NR, d0 + 1, pb);
+      weigh(b, p, pa, pb, v[0], v[1]);
+    });
+    if (!grid_sum<2, true, NT>(v, redS, S, k, epoch, [&]() {
+          S.step = S.step + 1;
+          new_state(S.step);
+        })) { finish(); return; }
+    mark(KK_COMBINE);
+    if (k.energy) {
+      if (!energy(S.step)) { finish(); return; }
+      mark(KK_ENERGY);
+    }
+  }
+  finish();
+}
+
+}  // namespace
+
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, bool fp64) {
+  const int nr = fp64 ? KCfg<double>::NR : KCfg<float>::NR;
+  const size_t rb = (rows + nr - 1) / nr;
+  return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 + (fp64 ? 0 : (size_t)(1 + 2 * n_groups) * 8) +
+         (size_t)n_groups * (fp64 ? 16 : 8) + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+}
+
+template <typename R, bool VEC>
+static cudaError_t prepare_t(size_t smem, int* ctas) {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, k_krylov<R, VEC>);
+  if (e != cudaSuccess) return e;
+  *ctas = 0;
+  if (smem + fa.sharedSizeBytes > 227 * 1024) return cudaSuccess;
+  e = cudaFuncSetAttribute(k_krylov<R, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_krylov<R, VEC>, KCfg<R>::NT, smem);
+}
+
+cudaError_t krylov_prepare(bool fp64, bool vec, size_t smem, int* ctas_per_sm) {
+  if (fp64) return prepare_t<double, false>(smem, ctas_per_sm);
+  return vec ? prepare_t<float, true>(smem, ctas_per_sm) : prepare_t<float, false>(smem, ctas_per_sm);
+}
+
+cudaError_t launch_krylov(bool fp64, bool vec, const KrylovArgs& k, int grid, size_t smem,
+                          cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(k.slots, 0, kKrylovSlotBytes, s);
+  if (e != cudaSuccess) return e;
+  void* args[] = {const_cast<KrylovArgs*>(&k)};
+  const void* f = fp64 ? (const void*)k_krylov<double, false>
+                  : vec ? (const void*)k_krylov<float, true>
+                        : (const void*)k_krylov<float, false>;
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(fp64 ? KCfg<double>::NT : KCfg<float>::NT),
+                                     args, smem, s);
+}
+
+}  // namespace ed
