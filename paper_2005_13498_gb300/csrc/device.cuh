@@ -96,6 +96,40 @@ __device__ __forceinline__ void block_reduce(double (&v)[K], double* red) {
   }
 }
 
+// Write this block's partials; the last block of [b0, b1) sums all partials
+// in block order.  Returns true in every thread of the last block; the totals
+// are valid in thread 0.
+template <int K>
+__device__ __forceinline__ bool reduce_last_block(double (&v)[K], int blk, int b0,
+                                                  int b1, double* partials,
+                                                  unsigned* counter,
+                                                  double* red, int* flag) {
+  block_reduce<K>(v, red);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) partials[(size_t)blk * K + k] = v[k];
+    __threadfence();
+    unsigned ticket = atomicAdd(counter, 1u);
+    *flag = (ticket == (unsigned)(b1 - b0 - 1));
+  }
+  __syncthreads();
+  if (!*flag) return false;
+  __threadfence();
+  double acc[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) acc[k] = 0.0;
+  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[k] += __ldcg(&partials[(size_t)b * K + k]);
+  block_reduce<K>(acc, red);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = acc[k];
+    *counter = 0u;
+  }
+  return true;
+}
+
 // Column pair (2p, 2p+1) of a row: one 16-byte access for aligned complex64
 // rows (VEC), else two element accesses with the second column checked.
 // STREAM: data read or written once in this pass (the previous Krylov vector,

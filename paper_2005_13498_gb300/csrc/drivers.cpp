@@ -96,17 +96,22 @@ struct GsApply {
   int nblk = 0;
 };
 
-// x, w: device buffers of length D the autotuner may read and overwrite.
-std::string gs_apply_setup(GsApply& G, ed_ctx* ctx, const double2* x, double2* w,
+// The products w = H v_i of the solve: v_i = V + i D for i < n (n - 1 Lanczos
+// vectors and the Ritz vector).  The autotuner may read V and overwrite w.
+std::string gs_apply_setup(GsApply& G, ed_ctx* ctx, const double2* x, int n, double2* w,
                            cudaStream_t s) {
   // hop-ordered down-spin tables: the Lanczos vectors keep their columns in
   // that order, and the result goes back to ascending-word order at the end
   std::vector<SectorDev> secs = {ctx->sec.dev_hop};
-  std::vector<VecDev> vd(1);
-  std::memset(vd.data(), 0, sizeof(VecDev));
-  vd[0].D = ctx->dim_up * ctx->dim_dn;
-  vd[0].x1 = const_cast<double2*>(x);
-  vd[0].w = w;
+  // one entry per source vector; a product takes its own (block maps name
+  // entry 0 of the pointer they are launched with)
+  std::vector<VecDev> vd(n);
+  std::memset(vd.data(), 0, sizeof(VecDev) * n);
+  for (int i = 0; i < n; ++i) {
+    vd[i].D = ctx->dim_up * ctx->dim_dn;
+    vd[i].x1 = const_cast<double2*>(x) + (size_t)i * vd[i].D;
+    vd[i].w = w;
+  }
   const int ng = 2 * ctx->lat.n_classes;
   std::vector<double> cf(std::max(1, ng) * 2, 0.0);
   const double A0[3] = {0, 0, 0};
@@ -147,6 +152,10 @@ std::string gs_apply_setup(GsApply& G, ed_ctx* ctx, const double2* x, double2* w
   std::string err = tune_apply(tt, s, &G.shape, &amap, &cmap);
   if (!err.empty()) return err;
   assign_apply_ranges(amap, G.shape.mv, vd.data(), 1);
+  for (int i = 1; i < n; ++i) {
+    vd[i].apply_begin = vd[0].apply_begin;
+    vd[i].apply_end = vd[0].apply_end;
+  }
   ED_TRY(upload(G.vec, vd));
   ED_TRY(upload(G.amap, amap));
   ED_TRY(upload(G.cmap, cmap));
@@ -161,18 +170,22 @@ std::string gs_apply_setup(GsApply& G, ed_ctx* ctx, const double2* x, double2* w
   return "";
 }
 
-cudaError_t gs_apply(GsApply& G, const double2* x, double2* w, cudaStream_t s) {
-  VecDev vd;
-  cudaError_t e = cudaMemcpyAsync(&vd, G.vec.p, sizeof(VecDev), cudaMemcpyDeviceToHost, s);
-  if (e != cudaSuccess) return e;
-  if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;
-  vd.x1 = const_cast<double2*>(x);
-  vd.w = w;
-  if ((e = cudaMemcpyAsync(G.vec.p, &vd, sizeof(VecDev), cudaMemcpyHostToDevice, s)) != cudaSuccess)
-    return e;
-  if ((e = launch_apply(true, G.args, G.nblk, G.shape, 0, s)) != cudaSuccess) return e;
-  return cudaStreamSynchronize(s);  // vd is a host temporary
+cudaError_t gs_apply(GsApply& G, int i, cudaStream_t s) {
+  BatchArgs a = G.args;
+  a.vec = G.args.vec + i;
+  return launch_apply(true, a, G.nblk, G.shape, 0, s);
 }
+
+// Pinned host memory and events of a solve's pipeline.
+struct GsHost {
+  double* p = nullptr;   // [kGsMaxVectors][2]: alpha_k, beta_k
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  ~GsHost() {
+    if (p) cudaFreeHost(p);
+    for (cudaEvent_t e : ev)
+      if (e) cudaEventDestroy(e);
+  }
+};
 
 }  // namespace
 
@@ -193,28 +206,38 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   // V holds K + 1 vectors, w and y one each
   if (ctx->workspace_limit > 0)
     kfit = std::min<int64_t>(kfit, ctx->workspace_limit / ((int64_t)D * 16) - 3);
-  int K = (int)std::min<int64_t>(std::min<int64_t>(200, kfit), D);
+  int K = (int)std::min<int64_t>(std::min<int64_t>(kGsMaxVectors, kfit), D);
   K = std::min(K, max_iter);
   if (K < 2 && D > 1)
     return fail(ctx, ED_ERR_OOM,
                 "not enough device memory (or workspace limit) for two Lanczos vectors");
   if (D == 1) K = 1;
-  DevMem V, w, y, part, red, cvec, cdev, sdev;
-  CK(ctx, V.alloc((size_t)(K + 1) * D * 16));
+  // V: K + 1 Lanczos vectors and the Ritz vector y
+  DevMem V, w, part, red, sdev, dots, coef, scal, phase;
+  CK(ctx, V.alloc((size_t)(K + 2) * D * 16));
   CK(ctx, w.alloc((size_t)D * 16));
-  CK(ctx, y.alloc((size_t)D * 16));
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(1216, (D + 2047) / 2048));
-  CK(ctx, part.alloc(sizeof(double2) * (size_t)nblk * (K + 1)));
-  CK(ctx, red.alloc(sizeof(double) * 2));
-  CK(ctx, cdev.alloc(sizeof(double2) * (K + 1)));
+  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(kGsMaxBlocks, (D + 2047) / 2048));
+  CK(ctx, part.alloc(sizeof(double) * 2 * kGsMaxBlocks));
+  CK(ctx, red.alloc(sizeof(double) * 2 + sizeof(unsigned)));
   CK(ctx, sdev.alloc(sizeof(double) * (K + 1)));
+  CK(ctx, dots.alloc(sizeof(double) * (size_t)gs_dot_blocks(D) * K));
+  CK(ctx, coef.alloc(sizeof(double) * K));
+  CK(ctx, scal.alloc(sizeof(GsScalars)));
+  CK(ctx, phase.alloc(kGsPhaseBlocks * (sizeof(double) + sizeof(int64_t))));
   GsApply G;
-  CKS(ctx, gs_apply_setup(G, ctx, static_cast<const double2*>(V.p),
+  CKS(ctx, gs_apply_setup(G, ctx, static_cast<const double2*>(V.p), K + 2,
                          static_cast<double2*>(w.p), s));
   double2* Vp = static_cast<double2*>(V.p);
   double2* wp = static_cast<double2*>(w.p);
-  double2* yp = static_cast<double2*>(y.p);
+  double2* yp = Vp + (size_t)(K + 1) * D;
   double* redp = static_cast<double*>(red.p);
+  unsigned* counter = reinterpret_cast<unsigned*>(redp + 2);
+  CK(ctx, cudaMemsetAsync(counter, 0, sizeof(unsigned), s));
+  GsScalars* sc_dev = static_cast<GsScalars*>(scal.p);
+  GsHost H;
+  CK(ctx, cudaHostAlloc(reinterpret_cast<void**>(&H.p), sizeof(double) * 2 * kGsMaxVectors,
+                        cudaHostAllocDefault));
+  for (cudaEvent_t& e : H.ev) CK(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   auto vk = [&](int k) { return Vp + (size_t)k * D; };
   auto norm_dot = [&](const double2* a, const double2* b, double out[2]) -> cudaError_t {
     cudaError_t e = launch_norm_dot(a, b, D, static_cast<double*>(part.p), nblk, redp, s);
@@ -222,6 +245,19 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
     e = cudaMemcpyAsync(out, redp, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return e;
     return cudaStreamSynchronize(s);
+  };
+  // Lanczos step k: everything on the stream, alpha_k and beta_k to the host
+  auto enqueue = [&](int k) -> cudaError_t {
+    cudaError_t e = gs_apply(G, k, s);
+    if (e == cudaSuccess)
+      e = launch_gs_step(Vp, D, k, wp, sc_dev, static_cast<double*>(dots.p),
+                         static_cast<double*>(coef.p), static_cast<double*>(part.p), counter,
+                         vk(k + 1), s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(H.p + 2 * k, sc_dev->alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(H.p + 2 * k + 1, sc_dev->beta + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaEventRecord(H.ev[k & 1], s) : e;
   };
   // seeded start vector, normalised
   CK(ctx, launch_random_fill(vk(0), D, seed, s));
@@ -236,41 +272,20 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   while (applies < max_iter && !converged) {
     al.clear();
     be.clear();
-    int k = 0;
-    for (; k < K; ++k) {
-      CK(ctx, gs_apply(G, vk(k), wp, s));
+    // step k + 1 is on the stream while the host examines step k; when step
+    // k turns out to be the last, the work of step k + 1 is discarded
+    CK(ctx, enqueue(0));
+    for (int k = 0; k < K; ++k) {
+      if (k + 1 < K) CK(ctx, enqueue(k + 1));
+      CK(ctx, cudaEventSynchronize(H.ev[k & 1]));
       ++applies;
-      CK(ctx, norm_dot(vk(k), wp, nd));
-      const double a = nd[1];
-      al.push_back(a);
-      double tmp = a;
-      CK(ctx, cudaMemcpyAsync(redp, &tmp, sizeof(double), cudaMemcpyHostToDevice, s));
-      CK(ctx, launch_axpy_real(wp, vk(k), D, redp, -1.0, s));
-      if (k > 0) {
-        double bprev = be.back();
-        CK(ctx, cudaMemcpyAsync(redp + 1, &bprev, sizeof(double), cudaMemcpyHostToDevice, s));
-        CK(ctx, launch_axpy_real(wp, vk(k - 1), D, redp + 1, -1.0, s));
-      }
-      // full reorthogonalisation, classical Gram-Schmidt applied twice
-      for (int pass = 0; pass < 2; ++pass) {
-        CK(ctx, launch_multidot(vk(0), D, k + 1, wp, D, static_cast<double2*>(part.p), nblk, s));
-        CK(ctx, launch_reduce_cols(static_cast<double2*>(part.p), nblk, k + 1,
-                                   static_cast<double2*>(cdev.p), s));
-        CK(ctx, launch_multiaxpy(vk(0), D, k + 1, static_cast<double2*>(cdev.p), wp, D, s));
-      }
-      CK(ctx, norm_dot(wp, nullptr, nd));
-      const double b = std::sqrt(nd[0]);
+      al.push_back(H.p[2 * k]);
+      const double b = H.p[2 * k + 1];
       be.push_back(b);
       lowest_eigenpair(al, be, &theta, sv);
       const double est = b * std::fabs(sv.back());
       const double sc = std::max(1.0, std::fabs(theta));
-      if (est <= 0.1 * tol * sc || b <= 1e-14 * sc || k + 1 == K || applies >= max_iter) {
-        ++k;
-        break;
-      }
-      CK(ctx, cudaMemcpyAsync(vk(k + 1), wp, (size_t)D * 16, cudaMemcpyDeviceToDevice, s));
-      CK(ctx, cudaMemcpyAsync(redp, &nd[0], sizeof(double), cudaMemcpyHostToDevice, s));
-      CK(ctx, launch_scale(vk(k + 1), D, redp, true, s));
+      if (est <= 0.1 * tol * sc || b <= 1e-14 * sc || k + 1 == K || applies >= max_iter) break;
     }
     // Ritz vector y = V s, normalised
     CK(ctx, cudaMemcpyAsync(sdev.p, sv.data(), sizeof(double) * sv.size(), cudaMemcpyHostToDevice, s));
@@ -279,7 +294,7 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
     CK(ctx, cudaMemcpyAsync(redp, &nd[0], sizeof(double), cudaMemcpyHostToDevice, s));
     CK(ctx, launch_scale(yp, D, redp, true, s));
     // true residual |H y - theta' y| with theta' = <y, H y>
-    CK(ctx, gs_apply(G, yp, wp, s));
+    CK(ctx, gs_apply(G, K + 1, s));
     ++applies;
     CK(ctx, norm_dot(yp, wp, nd));
     theta = nd[1];
@@ -292,26 +307,16 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
     // restart from the Ritz vector
     CK(ctx, cudaMemcpyAsync(vk(0), yp, (size_t)D * 16, cudaMemcpyDeviceToDevice, s));
   }
-  // columns back to ascending-word order, then the phase fix on the host:
+  // columns back to ascending-word order, then the phase fix: the
   // largest-magnitude element real and positive
   CK(ctx, launch_permute_cols(true, yp, (int)ctx->dim_up, (int)ctx->dim_dn,
                               static_cast<const int32_t*>(ctx->sec.dn_order.p), false, s));
-  std::vector<std::complex<double>> h(D);
-  CK(ctx, cudaMemcpyAsync(h.data(), yp, (size_t)D * 16, cudaMemcpyDeviceToHost, s));
+  const bool to_device = is_device_ptr(psi);
+  double2* out = to_device ? static_cast<double2*>(psi) : wp;
+  double* val = static_cast<double*>(phase.p);
+  CK(ctx, launch_gs_phase(yp, out, D, val, reinterpret_cast<int64_t*>(val + kGsPhaseBlocks), s));
+  if (!to_device) CK(ctx, cudaMemcpyAsync(psi, wp, (size_t)D * 16, cudaMemcpyDeviceToHost, s));
   CK(ctx, cudaStreamSynchronize(s));
-  int64_t kmax = 0;
-  double amax = -1.0;
-  for (int64_t i = 0; i < D; ++i) {
-    const double a = std::abs(h[i]);
-    if (a > amax) { amax = a; kmax = i; }
-  }
-  const std::complex<double> ph = std::conj(h[kmax]) / std::abs(h[kmax]);
-  for (auto& z : h) z *= ph;
-  h[kmax] = std::complex<double>(std::abs(h[kmax]), 0.0);
-  if (is_device_ptr(psi))
-    CK(ctx, cudaMemcpy(psi, h.data(), (size_t)D * 16, cudaMemcpyHostToDevice));
-  else
-    std::memcpy(psi, h.data(), (size_t)D * 16);
   *E0 = theta;
   if (resid_out) *resid_out = resid;
   if (!std::isfinite(theta) || !std::isfinite(resid))

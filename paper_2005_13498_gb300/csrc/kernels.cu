@@ -24,40 +24,6 @@
 
 namespace ed {
 
-// Write this block's partials; the last block of [b0, b1) sums all partials
-// in block order.  Returns true in every thread of the last block; the totals
-// are valid in thread 0.
-template <int K>
-__device__ __forceinline__ bool reduce_last_block(double (&v)[K], int blk, int b0,
-                                                  int b1, double* partials,
-                                                  unsigned* counter,
-                                                  double* red, int* flag) {
-  block_reduce<K>(v, red);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) partials[(size_t)blk * K + k] = v[k];
-    __threadfence();
-    unsigned ticket = atomicAdd(counter, 1u);
-    *flag = (ticket == (unsigned)(b1 - b0 - 1));
-  }
-  __syncthreads();
-  if (!*flag) return false;
-  __threadfence();
-  double acc[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = 0.0;
-  for (int b = b0 + threadIdx.x; b < b1; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[k] += __ldcg(&partials[(size_t)b * K + k]);
-  block_reduce<K>(acc, red);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = acc[k];
-    *counter = 0u;
-  }
-  return true;
-}
-
 // Whether the Lanczos passes of step j are skipped: after a breakdown, or
 // once the adaptive check of a step <= j - 2 has converged.  The check of
 // step j - 1 runs concurrently with pass j (its result must not change
@@ -1706,58 +1672,6 @@ __global__ void __launch_bounds__(256) k_transpose(const C* in, C* out, int rows
 }
 
 // ------------------------------------------------------ ground-state helpers
-__global__ void __launch_bounds__(256)
-k_multidot(const double2* V, int64_t ldV, int k, const double2* w, int64_t D,
-           double2* partial) {
-  // block b handles chunk [b*chunk, (b+1)*chunk); partial[b*k + i]
-  extern __shared__ double2 sacc[];  // [blockDim/32][k]
-  const int64_t chunk = (D + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = blockIdx.x * chunk, i1 = min(D, i0 + chunk);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int i = 0; i < k; ++i) {
-    double re = 0.0, im = 0.0;
-    const double2* Vi = V + (size_t)i * ldV;
-    for (int64_t t = i0 + threadIdx.x; t < i1; t += blockDim.x) {
-      const double2 a = Vi[t], b = w[t];
-      re += a.x * b.x + a.y * b.y;
-      im += a.x * b.y - a.y * b.x;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      re += __shfl_down_sync(0xffffffffu, re, o);
-      im += __shfl_down_sync(0xffffffffu, im, o);
-    }
-    if (lane == 0) sacc[wid * k + i] = make_double2(re, im);
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    double re = 0.0, im = 0.0;
-    for (int q = 0; q < nw; ++q) { re += sacc[q * k + i].x; im += sacc[q * k + i].y; }
-    partial[(size_t)blockIdx.x * k + i] = make_double2(re, im);
-  }
-}
-
-__global__ void k_reduce_cols(const double2* partial, int nblk, int k, double2* out) {
-  for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < k; i += blockDim.x * gridDim.x) {
-    double re = 0.0, im = 0.0;
-    for (int b = 0; b < nblk; ++b) { re += partial[(size_t)b * k + i].x; im += partial[(size_t)b * k + i].y; }
-    out[i] = make_double2(re, im);
-  }
-}
-
-__global__ void k_multiaxpy(const double2* V, int64_t ldV, int k, const double2* c,
-                            double2* w, int64_t D) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < D;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    double2 acc = w[t];
-    for (int i = 0; i < k; ++i) {
-      const double2 v = V[(size_t)i * ldV + t], ci = c[i];
-      acc.x -= ci.x * v.x - ci.y * v.y;
-      acc.y -= ci.x * v.y + ci.y * v.x;
-    }
-    w[t] = acc;
-  }
-}
-
 __global__ void k_combine_real(const double2* V, int64_t ldV, int k, const double* c,
                                double2* y, int64_t D) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < D;
@@ -2230,30 +2144,6 @@ cudaError_t launch_transpose(bool fp64, const void* in, void* out, int rows, int
   else
     k_transpose<float2><<<grid, 256, 0, s>>>(static_cast<const float2*>(in),
                                              static_cast<float2*>(out), rows, cols);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_multidot(const double2* V, int64_t ldV, int k, const double2* w,
-                            int64_t D, double2* partial, int nblk, cudaStream_t s) {
-  const size_t sm = (size_t)(256 / 32) * k * sizeof(double2);
-  if (sm > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_multidot, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
-    if (e != cudaSuccess) return e;
-  }
-  k_multidot<<<nblk, 256, sm, s>>>(V, ldV, k, w, D, partial);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_reduce_cols(const double2* partial, int nblk, int k, double2* out,
-                               cudaStream_t s) {
-  k_reduce_cols<<<(k + 127) / 128, 128, 0, s>>>(partial, nblk, k, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_multiaxpy(const double2* V, int64_t ldV, int k, const double2* c,
-                             double2* w, int64_t D, cudaStream_t s) {
-  k_multiaxpy<<<grid_for(D, 256), 256, 0, s>>>(V, ldV, k, c, w, D);
   return cudaGetLastError();
 }
 

@@ -211,16 +211,28 @@ cudaError_t launch_krylov(bool fp64, bool vec, const KrylovArgs& k, int grid, si
                           cudaStream_t s);
 
 // ---- ground-state helpers (float64 only) ---------------------------------
-// partial[blk][i] = sum over block chunk of conj(V_i) w, i < k  (k <= 256)
-cudaError_t launch_multidot(const double2* V, int64_t ldV, int k,
-                            const double2* w, int64_t D, double2* partial,
-                            int nblk, cudaStream_t s);
-cudaError_t launch_reduce_cols(const double2* partial, int nblk, int k,
-                               double2* out, cudaStream_t s);
-// w -= sum_i c_i V_i  (c on device)
-cudaError_t launch_multiaxpy(const double2* V, int64_t ldV, int k,
-                             const double2* c, double2* w, int64_t D,
-                             cudaStream_t s);
+// Scalars of the ground-state Lanczos recursion on the device.
+constexpr int kGsMaxVectors = 200;   // Krylov vectors per restart
+constexpr int kGsMaxBlocks = 1216;   // blocks of the elementwise kernels
+constexpr int kGsPhaseBlocks = 256;
+struct GsScalars {
+  double alpha[kGsMaxVectors], beta[kGsMaxVectors];
+  double before, norm2;   // |w|^2 before the projections, and after
+  int again;              // whether the next projection pass runs
+};
+// Blocks (rows of `dots`) of the projection kernel for vectors of D elements.
+int64_t gs_dot_blocks(int64_t D);
+// The rest of Lanczos step k after w = H v_k (ground.cu): alpha_k, the
+// three-term recursion, the projection against v_0 .. v_k (V: vectors of D
+// elements back to back), beta_k and vnext = v_{k+1}.  dots: gs_dot_blocks(D)
+// x (k + 1) doubles, coef: k + 1, partials: kGsMaxBlocks, counter: one zero.
+cudaError_t launch_gs_step(const double2* V, int64_t D, int k, double2* w, GsScalars* S,
+                           double* dots, double* coef, double* partials, unsigned* counter,
+                           double2* vnext, cudaStream_t s);
+// out = y times the phase that makes its largest element (the first of the
+// largest) real and positive; val, idx: kGsPhaseBlocks entries of scratch.
+cudaError_t launch_gs_phase(const double2* y, double2* out, int64_t D, double* val, int64_t* idx,
+                            cudaStream_t s);
 // y = sum_i c_i V_i (c real, on device)
 cudaError_t launch_combine_real(const double2* V, int64_t ldV, int k,
                                 const double* c, double2* y, int64_t D,
