@@ -405,7 +405,7 @@ ed_status ed_device_bytes(const ed_ctx* ctx, int64_t* bytes) {
               S.dn_ellp32.bytes + S.dn_ellpr.bytes + S.dnh_off.bytes + S.dnh_ent.bytes +
               S.dnh_word.bytes + S.dnh_eps.bytes + S.dnh_tslot_off.bytes +
               S.dnh_slot_grp.bytes + S.dnh_ellp32.bytes + S.dnh_ellpr.bytes +
-              S.dn_order.bytes;
+              S.dn_order.bytes + ctx->docc.bytes;
   if (ctx->engine) b += ctx->engine->device_bytes();
   if (ctx->spec_engine) b += ctx->spec_engine->device_bytes();
   *bytes = b;
@@ -763,24 +763,23 @@ ed_status ed_double_occupation(ed_ctx* ctx, const void* psi, ed_dtype dtype, dou
   const int64_t D = ctx->dim_up * ctx->dim_dn;
   const size_t esz = fp64 ? 16 : 8;
   cudaStream_t s = ctx->stream;
-  DevMem tmp, part, out;
+  DevMem tmp;
   const void* p = psi;
   if (!is_device_ptr(psi)) {
     CK(ctx, tmp.alloc(D * esz));
     CK(ctx, cudaMemcpyAsync(tmp.p, psi, D * esz, cudaMemcpyHostToDevice, s));
     p = tmp.p;
   }
-  const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(1216, (D + 1023) / 1024));
-  CK(ctx, part.alloc(sizeof(double) * (kMaxSites + 1) * nblk));
-  CK(ctx, out.alloc(sizeof(double) * (kMaxSites + 1)));
-  CK(ctx, launch_docc_sites(fp64, p, &ctx->sec.dev, (int)ctx->dim_up, (int)ctx->dim_dn, ctx->Ns,
-                            static_cast<double*>(part.p), nblk, static_cast<double*>(out.p), s));
-  double h[kMaxSites + 1];
-  CK(ctx, cudaMemcpyAsync(h, out.p, sizeof(h), cudaMemcpyDeviceToHost, s));
+  if (!ctx->docc.p) CK(ctx, ctx->docc.alloc(kDoccScratchDoubles * sizeof(double)));
+  double* scratch = static_cast<double*>(ctx->docc.p);
+  CK(ctx, launch_docc_sites(fp64, p, ctx->sec.dev, scratch, s));
+  double h[kDoccVals];
+  CK(ctx, cudaMemcpyAsync(h, scratch + kDoccScratchDoubles - kDoccVals, sizeof(h),
+                          cudaMemcpyDeviceToHost, s));
   CK(ctx, cudaStreamSynchronize(s));
-  *d_avg = h[0] / ctx->Ns;
+  *d_avg = docc_average(h, ctx->Ns);
   if (d_site)
-    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[1 + i];
+    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[i];
   return ED_OK;
 }
 

@@ -64,6 +64,7 @@ struct ed_ctx {
   std::string err;
   cudaStream_t stream = nullptr;
   int device = 0;
+  ed::DevMem docc;   // scratch of ed_double_occupation, kept between calls
   ed::ApplyPlan plan;
   std::unique_ptr<ed::Engine> engine;
   std::unique_ptr<ed::Engine> spec_engine;

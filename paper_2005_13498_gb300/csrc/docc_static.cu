@@ -10,20 +10,19 @@
 #include <mutex>
 
 #include "ctx.h"
+#include "docc.cuh"
 
 namespace ed {
 
 namespace {
 
-constexpr int kStaticSlots = kMaxSites + 1;          // total + one per site
-constexpr int kStaticBlocks = 1024;                   // per-block partial rows
-constexpr int64_t kStaticChunk = 65536;               // elements per block
-constexpr int64_t kStaticMaxElems = kStaticChunk * kStaticBlocks;  // 67,108,864
+constexpr int64_t kStaticMaxElems = 67108864;
 constexpr int kStaticMaxDevices = 64;
 
-// Partial sums of every block (kStaticBlocks rows) followed by the final
-// sums (one row): (1024 + 1) * 17 doubles = 139,400 bytes per device.
-__device__ __align__(256) double g_docc_scratch[(kStaticBlocks + 1) * kStaticSlots];
+// Partial sums of every block (1024 rows of 17 doubles) followed by the
+// final sums (one row): 139,400 bytes per device.
+static_assert(kDoccScratchDoubles * sizeof(double) == 139400, "the documented size");
+__device__ __align__(256) double g_docc_scratch[kDoccScratchDoubles];
 
 std::mutex g_scratch_mutex;
 double* g_scratch_ptr[kStaticMaxDevices] = {nullptr};
@@ -45,51 +44,6 @@ cudaError_t scratch_address(double** out) {
   }
   *out = g_scratch_ptr[dev];
   return cudaSuccess;
-}
-
-template <typename C>
-__global__ void __launch_bounds__(256)
-k_docc_sites_static(const C* psi, SectorDev sd, double* scratch) {
-  __shared__ double red[32][kStaticSlots];
-  const int64_t D = (int64_t)sd.dim_up * sd.dim_dn;
-  const int64_t i0 = blockIdx.x * kStaticChunk;
-  const int64_t i1 = i0 + kStaticChunk < D ? i0 + kStaticChunk : D;
-  double v[kStaticSlots];
-#pragma unroll
-  for (int i = 0; i < kStaticSlots; ++i) v[i] = 0.0;
-  for (int64_t t = i0 + threadIdx.x; t < i1; t += blockDim.x) {
-    const int u = (int)(t / sd.dim_dn);
-    const int d = (int)(t - (int64_t)u * sd.dim_dn);
-    const C p = psi[t];
-    const double q = (double)p.x * p.x + (double)p.y * p.y;
-    const uint32_t both = sd.up_word[u] & sd.dn_word[d];
-    v[0] += __popc(both) * q;
-#pragma unroll
-    for (int i = 0; i < kMaxSites; ++i)
-      if ((both >> i) & 1u) v[1 + i] += q;
-  }
-  // warp sums, then one warp sums the warps in a fixed order
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < kStaticSlots; ++i) {
-    double s = v[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if (lane == 0) red[wid][i] = s;
-  }
-  __syncthreads();
-  if (threadIdx.x < kStaticSlots) {
-    double s = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w][threadIdx.x];
-    scratch[(size_t)blockIdx.x * kStaticSlots + threadIdx.x] = s;   // every slot rewritten
-  }
-}
-
-__global__ void k_docc_sum_static(double* scratch, int nblk) {
-  const int i = threadIdx.x;
-  if (i >= kStaticSlots) return;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += scratch[(size_t)b * kStaticSlots + i];
-  scratch[(size_t)kStaticBlocks * kStaticSlots + i] = s;
 }
 
 }  // namespace
@@ -118,22 +72,13 @@ extern "C" ed_status ed_double_occupation_static(ed_ctx* ctx, const void* psi, e
   double* scratch = nullptr;
   CK(ctx, scratch_address(&scratch));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int nblk = (int)((D + kStaticChunk - 1) / kStaticChunk);
-  if (dtype == ED_C128)
-    k_docc_sites_static<double2><<<nblk, 256, 0, s>>>(static_cast<const double2*>(psi),
-                                                       ctx->sec.dev, scratch);
-  else
-    k_docc_sites_static<float2><<<nblk, 256, 0, s>>>(static_cast<const float2*>(psi),
-                                                      ctx->sec.dev, scratch);
-  CK(ctx, cudaGetLastError());
-  k_docc_sum_static<<<1, 32, 0, s>>>(scratch, nblk);
-  CK(ctx, cudaGetLastError());
-  double h[kStaticSlots];
-  CK(ctx, cudaMemcpyAsync(h, scratch + (size_t)kStaticBlocks * kStaticSlots, sizeof(h),
+  CK(ctx, launch_docc(dtype == ED_C128, psi, ctx->sec.dev, scratch, s));
+  double h[kDoccVals];
+  CK(ctx, cudaMemcpyAsync(h, scratch + kDoccScratchDoubles - kDoccVals, sizeof(h),
                           cudaMemcpyDeviceToHost, s));
   CK(ctx, cudaStreamSynchronize(s));
-  *d_avg = h[0] / ctx->Ns;
+  *d_avg = docc_average(h, ctx->Ns);
   if (d_site)
-    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[1 + i];
+    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[i];
   return ED_OK;
 }

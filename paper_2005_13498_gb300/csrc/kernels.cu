@@ -19,6 +19,7 @@
 // Reductions are deterministic: per-block partial sums in float64, then the
 // last block of each vector sums the partials in block order.
 #include "device.cuh"
+#include "docc.cuh"
 
 #include <cstdio>
 
@@ -1746,40 +1747,6 @@ __global__ void k_random_fill(double2* x, int64_t D, uint64_t seed) {
   }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(256)
-k_docc_sites(const typename C2T<R>::T* psi, SectorDev sd, int Ns, double* partial) {
-  __shared__ double red[32 * (kMaxSites + 1)];
-  const int64_t D = (int64_t)sd.dim_up * sd.dim_dn;
-  const int64_t chunk = (D + gridDim.x - 1) / gridDim.x;
-  const int64_t i0 = blockIdx.x * chunk, i1 = min(D, i0 + chunk);
-  double v[kMaxSites + 1];
-#pragma unroll
-  for (int i = 0; i <= kMaxSites; ++i) v[i] = 0.0;
-  for (int64_t t = i0 + threadIdx.x; t < i1; t += blockDim.x) {
-    const int u = (int)((uint32_t)t / (uint32_t)sd.dim_dn);
-    const int d = (int)((uint32_t)t - (uint32_t)u * (uint32_t)sd.dim_dn);
-    const auto p = psi[t];
-    const double q = (double)p.x * p.x + (double)p.y * p.y;
-    const uint32_t both = sd.up_word[u] & sd.dn_word[d];
-    v[0] += __popc(both) * q;
-#pragma unroll
-    for (int i = 0; i < kMaxSites; ++i)
-      if ((both >> i) & 1u) v[1 + i] += q;
-  }
-  block_reduce<kMaxSites + 1>(v, red);
-  if (threadIdx.x == 0)
-    for (int i = 0; i <= kMaxSites; ++i) partial[(size_t)blockIdx.x * (kMaxSites + 1) + i] = v[i];
-}
-
-__global__ void k_sum_sites(const double* partial, int nblk, int K, double* out) {
-  const int i = threadIdx.x;
-  if (i >= K) return;
-  double s = 0.0;
-  for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * K + i];
-  out[i] = s;
-}
-
 __global__ void k_convert_c128_c64(const double2* in, float2* out, int64_t n) {
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n;
        t += (int64_t)gridDim.x * blockDim.x)
@@ -2177,19 +2144,9 @@ cudaError_t launch_random_fill(double2* x, int64_t D, uint64_t seed, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_docc_sites(bool fp64, const void* psi, const SectorDev* sec, int dim_up,
-                              int dim_dn, int Ns, double* partial, int nblk, double* out,
+cudaError_t launch_docc_sites(bool fp64, const void* psi, const SectorDev& sec, double* scratch,
                               cudaStream_t s) {
-  (void)dim_up;
-  (void)dim_dn;
-  if (fp64)
-    k_docc_sites<double><<<nblk, 256, 0, s>>>(static_cast<const double2*>(psi), *sec, Ns,
-                                              partial);
-  else
-    k_docc_sites<float><<<nblk, 256, 0, s>>>(static_cast<const float2*>(psi), *sec, Ns,
-                                             partial);
-  k_sum_sites<<<1, 32, 0, s>>>(partial, nblk, kMaxSites + 1, out);
-  return cudaGetLastError();
+  return launch_docc(fp64, psi, sec, scratch, s);
 }
 
 cudaError_t launch_convert(const void* in, bool in_fp64, void* out, bool out_fp64,

@@ -23,7 +23,7 @@ CASES = [
     (synth.chain(3), 0, 2, 0, 0),        # three elements
     (synth.chain(5), 2, 1, 0, 0),        # 50 elements: part of one block
     (synth.ring(8), 4, 3, 0, 0),         # 3920 elements: chunks of 1024 with a remainder
-    (synth.ring(8), 4, 3, 0, 8),         # restarts with five Lanczos vectors
+    (synth.ring(8), 4, 3, 0, 23),        # restarts with 20 Lanczos vectors
     (synth.torus(3, 3), 4, 5, 1, 0),     # 15876 elements, result in host memory
 ]
 
