@@ -287,6 +287,135 @@ struct TileIO {
   }
 };
 
+// Comparisons of finite float64 values on the integer units (a float64
+// comparison takes a slot of the FP64 pipe).
+__device__ __forceinline__ bool is_zero(double a) {
+  return (__double_as_longlong(a) << 1) == 0;
+}
+__device__ __forceinline__ bool same(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b) || (is_zero(a) && is_zero(b));
+}
+
+// The off-diagonal part of H x for one row of Psi and the 64 columns of ELL
+// tile t, complex128: acc[h] of column 2 p + h of the lane's pair p (pcl: p
+// clamped to the row).  get(e): entry e < ne of the row's T_up list (source
+// row's element offset; group | sign << 31), sorted by group.
+//
+// FP64-pipe bound (a warp instruction occupies the SM's pipe for 16 cycles),
+// so the operations count: T_dn slots and T_up entries of one bond group share
+// one signed sum, a group whose coefficient equals the previous one's joins
+// its sum (the two directions of a bond that carries no phase; every bond at
+// A = 0), and a real coefficient costs half a complex product.  On the 2x7
+// ladder that is 75 operations per element where sums and products per group
+// and direction took 104: Lanczos pass 1.95 -> 1.55 ms (90 % of the pipe), the
+// step 65.6 -> 52.2 ms with the update.  With the T_up additions and the
+// products selected by short conditional blocks the compiler predicated them,
+// and switched-off instructions take the pipe's time as well: 1.94 ms.
+// lo, hi: which of the lane's two columns to compute
+// (uniform over the warp).
+__device__ __forceinline__ void ldcg2(const double2* row, int p, int dim, double2& v0, double2& v1) {
+  v0 = __ldcg(row + 2 * p);
+  v1 = czero<double2>();
+  if (2 * p + 1 < dim) v1 = __ldcg(row + 2 * p + 1);
+}
+
+template <typename Get>
+__device__ __forceinline__ void off_diagonal_c128(const SectorDev& sd, const double2* tile, int t,
+                                                  int pcl, const double2* x, int ne, Get&& get,
+                                                  const double2* coefS, bool lo, bool hi,
+                                                  double2 (&acc)[2]) {
+  using C = double2;
+  using TIO = TileIO<C, 1>;
+  const int lane = threadIdx.x & 31;
+  const int dim_dn = sd.dim_dn;
+  const uint32_t* ellp = TIO::ellp_for(sd.dn_ellp32, sd.dn_ellpr) + lane;
+  int q = __ldg(sd.dn_tslot_off + t), e = 0;
+  const int q1 = __ldg(sd.dn_tslot_off + t + 1);
+  constexpr uint32_t kEnd = 0xFFFFu;
+  uint32_t word = 0u, gq = kEnd;
+  if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
+  uint32_t ge = e < ne ? get(e).y & 0xFFu : kEnd;
+  C s0 = czero<C>(), s1 = s0, cur = s0;
+  acc[0] = acc[1] = s0;
+  auto flush = [&]() {
+    if (lo) { acc[0].x += cur.x * s0.x; acc[0].y += cur.x * s0.y; }
+    if (hi) { acc[1].x += cur.x * s1.x; acc[1].y += cur.x * s1.y; }
+    if (!is_zero(cur.y)) {   // uniform over the block
+      if (lo) { acc[0].x -= cur.y * s0.y; acc[0].y += cur.y * s0.x; }
+      if (hi) { acc[1].x -= cur.y * s1.y; acc[1].y += cur.y * s1.x; }
+    }
+  };
+  bool any = false;
+  for (;;) {
+    const uint32_t g = min(gq, ge);   // uniform over the warp
+    if (g == kEnd) break;
+    const C c = coefS[g];
+    if (!any) {
+      cur = c;
+      any = true;
+    } else if (!(same(c.x, cur.x) && same(c.y, cur.y))) {
+      flush();
+      s0 = s1 = czero<C>();
+      cur = c;
+    }
+    // the group's first T_up rows load while its T_dn slots are gathered
+    constexpr int NB = 4;
+    C v[NB][2];
+    double sg[NB];
+    int nb = 0;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+      if (nb == i && e + i < ne) {
+        const uint2 m = get(e + i);
+        if ((m.y & 0xFFu) == g) {
+          ldcg2(x + m.x, pcl, dim_dn, v[i][0], v[i][1]);
+          sg[i] = (m.y >> 31) ? -1.0 : 1.0;
+          nb = i + 1;
+        }
+      }
+    }
+    while (gq == g) {
+      const uint32_t w = word;
+      ++q;
+      if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
+      else gq = kEnd;
+      uint32_t o0, o1;
+      double g0, g1;
+      TIO::unpack<double>(w, o0, o1, g0, g1);
+      C a0[1], a1[1];
+      TIO::load_off(tile, o0, a0);
+      TIO::load_off(tile, o1, a1);
+      if (lo) cax(s0, g0, a0[0]);
+      if (hi) cax(s1, g1, a1[0]);
+    }
+    // one branch per count: short conditional blocks become predicated
+    // instructions, and those take the pipe's time also when switched off
+    auto add = [&](int i) {
+      if (lo) cax(s0, sg[i], v[i][0]);
+      if (hi) cax(s1, sg[i], v[i][1]);
+    };
+    switch (nb) {
+      case 1: add(0); break;
+      case 2: add(0); add(1); break;
+      case 3: add(0); add(1); add(2); break;
+      case 4: add(0); add(1); add(2); add(3); break;
+      default: break;
+    }
+    e += nb;
+    while (e < ne && (get(e).y & 0xFFu) == g) {
+      const uint2 m = get(e);
+      C u0, u1;
+      ldcg2(x + m.x, pcl, dim_dn, u0, u1);
+      const double s = (m.y >> 31) ? -1.0 : 1.0;
+      if (lo) cax(s0, s, u0);
+      if (hi) cax(s1, s, u1);
+      ++e;
+    }
+    ge = e < ne ? get(e).y & 0xFFu : kEnd;
+  }
+  if (any) flush();
+}
+
 // -------------------------------------------------------------------- expm
 // 1/k for the Taylor coefficients (evaluated by the compiler)
 struct InvK {

@@ -384,6 +384,12 @@ k_apply(BatchArgs a, int j) {
   using TIO = TileIO<C, NR>;
   constexpr int T = NT;                      // consumer threads (all threads without TMA)
   constexpr uint32_t kSlotBytes = (uint32_t)(T * PP * 2 * sizeof(C));   // one chunk of a row
+  // complex128, one row per CTA, one kernel: T_dn and T_up in one walk by bond
+  // group (off_diagonal_c128)
+  constexpr bool LEAN = sizeof(R) == 8 && NR == 1 && PP == 1 && !SPLIT && !TMA && !MV;
+  constexpr int kLean = LEAN ? 128 : 1;   // T_up entries of the row kept in shared memory
+  __shared__ uint2 upl[kLean];
+  __shared__ R utab[LEAN ? kMaxSites + 1 : 1];   // U n
   static_assert(!(TMA && SPLIT), "the TMA ring serves the one-kernel T_up");
   static_assert(!MV || (!TMA && !SPLIT), "multi-vector blocks use the one-kernel gathers");
   static_assert((NT / 32 + (TMA ? 1 : 0)) * (MV ? NR : 1) <= 64, "reduction scratch");
@@ -513,6 +519,17 @@ k_apply(BatchArgs a, int j) {
       TIO::store(tile, d, v);
     }
   }
+  int ue0 = 0, une = 0;
+  if constexpr (LEAN) {
+    ue0 = __ldg(sd.up_off + urow[0]);
+    une = __ldg(sd.up_off + urow[0] + 1) - ue0;
+    if (tid <= kMaxSites) utab[LEAN ? tid : 0] = (R)a.U * (R)tid;
+    for (int i = tid; i < min(une, kLean); i += T) {
+      const uint32_t en = __ldg(sd.up_ent + ue0 + i);
+      upl[i] = make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
+                          ((en >> kEntGroupShift) & 0xFFu) | (en & kEntSignBit));
+    }
+  }
   uint32_t uw[NR];
   R eu[NR];
 #pragma unroll
@@ -588,8 +605,19 @@ k_apply(BatchArgs a, int j) {
     // are read two at a time (tiles hold even slot counts).  The entries are
     // loaded two iterations (four slots) ahead of their gathers: the ELL
     // does not stay in L1, and its L2 latency was the exposed one
+    if constexpr (LEAN) {
+      if (pc + (tid - lane) < npairs)   // uniform over the warp
+        off_diagonal_c128(sd, tile, (pc + (tid - lane)) >> 5, min(pc + tid, npairs - 1), x, une,
+                          [&](int e) {
+                            if (e < kLean) return upl[e];   // uniform over the warp
+                            const uint32_t en = __ldg(sd.up_ent + ue0 + e);
+                            return make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
+                                              ((en >> kEntGroupShift) & 0xFFu) | (en & kEntSignBit));
+                          },
+                          coefS, true, true, acc[0]);
+    }
 #pragma unroll
-    for (int k = 0; k < PP; ++k) {
+    for (int k = 0; k < (LEAN ? 0 : PP); ++k) {
       const int pw0 = pc + (tid - lane) + k * T;     // first pair of the warp
       if (pw0 < npairs) {                             // uniform over the warp
         const int tw = pw0 >> 5;
@@ -755,7 +783,7 @@ k_apply(BatchArgs a, int j) {
       else
         tup_chunk_mv<R, NR, PP, 1, VEC, NT>(sd, xr, coefS, coefQ, urow[0], nrows, pc, npairs,
                                              dim_dn, acc);
-    } else if constexpr (!SPLIT && !TMA) {
+    } else if constexpr (!SPLIT && !TMA && !LEAN) {
       if (PP > 1 && pc + (PP - 1) * T < npairs)
         tup_chunk<R, NR, PP, PP, VEC, NT>(sd, x, coefS, coefQ, urow, nrows, pc, npairs, dim_dn, acc);
       else
@@ -795,8 +823,15 @@ k_apply(BatchArgs a, int j) {
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
           if (r < nrows) {
-            const R g0 = U * (R)__popc(uw[r] & dw0) + eu[r] + de0;
-            const R g1 = U * (R)__popc(uw[r] & dw1) + eu[r] + de1;
+            R g0, g1;
+            if constexpr (LEAN) {   // no conversions and products on the FP64 pipe
+              g0 = utab[__popc(uw[r] & dw0)];
+              g1 = utab[__popc(uw[r] & dw1)];
+              if (sd.up_eps) { g0 += eu[r] + de0; g1 += eu[r] + de1; }
+            } else {
+              g0 = U * (R)__popc(uw[r] & dw0) + eu[r] + de0;
+              g1 = U * (R)__popc(uw[r] & dw1) + eu[r] + de1;
+            }
             C a0 = acc[r][2 * k], a1 = acc[r][2 * k + 1];
             a0.x += g0 * xa[r].x;
             a0.y += g0 * xa[r].y;
@@ -1128,7 +1163,33 @@ __global__ void __launch_bounds__(256, 4) k_update(BatchArgs a, int j) {
   const void* px = xptr(vd, j, sizeof(C));
   const void* pxn = xptr(vd, j + 1, sizeof(C));
   const bool aligned = (((uintptr_t)pw | (uintptr_t)px | (uintptr_t)pxn) & 15u) == 0;
-  if (PAIR && aligned && (eb.begin & 1) == 0 && (eb.end & 1) == 0) {
+  if constexpr (sizeof(R) == 8) {
+    // complex128: an element per 16-byte access, four of each vector in flight
+    // per thread: 148 -> 101 us at Ns = 14 (5.6 TB/s)
+    const double2* w = static_cast<const double2*>(pw);
+    const double2* x = static_cast<const double2*>(px);
+    double2* xn = static_cast<double2*>(const_cast<void*>(pxn));
+    const int bd = blockDim.x;
+    for (int64_t i0 = eb.begin + threadIdx.x; i0 < eb.end; i0 += 4 * (int64_t)bd) {
+      double2 wv[4], xv[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t i = i0 + (int64_t)q * bd;
+        wv[q] = xv[q] = make_double2(0.0, 0.0);
+        if (i < eb.end) { wv[q] = __ldcs(w + i); xv[q] = __ldcs(x + i); }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int64_t i = i0 + (int64_t)q * bd;
+        double2 o;
+        o.x = wv[q].x - as * xv[q].x;
+        o.y = wv[q].y - as * xv[q].y;
+        if (i < eb.end) xn[i] = o;
+        nrm_d += o.x * o.x;
+        nrm_d += o.y * o.y;
+      }
+    }
+  } else if (PAIR && aligned && (eb.begin & 1) == 0 && (eb.end & 1) == 0) {
     const float4* w = static_cast<const float4*>(pw);
     const float4* x = static_cast<const float4*>(px);
     float4* xn = static_cast<float4*>(const_cast<void*>(pxn));
@@ -1799,6 +1860,7 @@ static const ApplyCfg kApplyCfgs[] = {
     // row of nr vectors per CTA (the per-vector pointers and sums need more
     // registers than configuration 1's three CTAs per SM allow)
     {false, 2, 2, 2, false, 0, 0, 0, 0, 0, 256, true}, {true, 2, 1, 2, false, 0, 0, 0, 0, 0, 256, true},
+    {true, 1, 1, 3, false, 0, 0, 0, 0},
 };
 static const int kNumApplyCfgs = (int)(sizeof(kApplyCfgs) / sizeof(kApplyCfgs[0]));
 
@@ -1957,7 +2019,8 @@ static cudaError_t prepare_apply_t(const LaunchShape& sh) {
   X(20, float, 1, 1, 2, true, 2, 3, 0, 256, 0, 512, false)   \
   X(21, float, 2, 1, 1, true, 2, 3, 0, 256, 0, 1024, false) \
   X(22, float, 2, 2, 2, false, 1, 1, 32, 256, 0, 256, true)  \
-  X(23, double, 2, 1, 2, false, 1, 1, 32, 256, 0, 256, true)
+  X(23, double, 2, 1, 2, false, 1, 1, 32, 256, 0, 256, true) \
+  X(24, double, 1, 1, 3, false, 1, 1, 32, 256, 0, 256, false)
 
 cudaError_t prepare_apply(bool fp64, const LaunchShape& sh) {
   (void)fp64;

@@ -192,9 +192,6 @@ __device__ __forceinline__ void ldcg_pair(const C* row, int p, int dim, C& v0, C
   }
 }
 
-template <typename C>
-__device__ __forceinline__ bool same(C a, C b) { return a.x == b.x && a.y == b.y; }
-
 // The off-diagonal part of H x for one item, NR tile rows x 64 columns (two
 // columns per lane): acc[r][h] of row r and column 2 p + h.
 //  complex64: T_dn over the ELL slots of the tile (two slots per turn, words
@@ -299,102 +296,14 @@ __device__ __forceinline__ void off_diagonal(
   }
 }
 
-//  complex128: FP64-pipe bound (a warp instruction occupies it for 16 cycles
-//  of the SM), so the operations count: T_dn slots and T_up entries of one
-//  bond group share one signed sum, a group whose coefficient equals the
-//  previous one's joins its sum, and a real coefficient costs half a complex
-//  product.  Per element of the 12-site torus that is 75 operations where
-//  separate sums with a product per group and direction take 104.  lo, hi:
-//  which of the lane's two columns the item covers (uniform over the warp).
+//  complex128: off_diagonal_c128 (device.cuh)
 __device__ __forceinline__ void off_diagonal(
     const SectorDev& sd, const double2* tile, int t, int p, int pcl, int npairs, const double2* x,
     const uint2* const (&list)[1], const int (&deg)[1], const double2* coefS, const float2*,
     bool, bool lo, bool hi, double2 (&acc)[1][2]) {
-  using C = double2;
-  using TIO = TileIO<C, 1>;
-  const int lane = threadIdx.x & 31;
-  const int dim_dn = sd.dim_dn;
-  const uint32_t* ellp = TIO::ellp_for(sd.dn_ellp32, sd.dn_ellpr) + lane;
   const uint2* lst = list[0];
-  const int ne = deg[0];
-  int q = __ldg(sd.dn_tslot_off + t), e = 0;
-  const int q1 = __ldg(sd.dn_tslot_off + t + 1);
-  constexpr uint32_t kEnd = 0xFFFFu;
-  uint32_t word = 0u, gq = kEnd;
-  if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
-  uint32_t ge = e < ne ? lst[e].y & 0xFFu : kEnd;
-  C s0 = czero<C>(), s1 = s0, cur = s0;
-  acc[0][0] = acc[0][1] = s0;
-  auto flush = [&]() {
-    if (cur.y == 0.0) {   // uniform over the block
-      if (lo) { acc[0][0].x += cur.x * s0.x; acc[0][0].y += cur.x * s0.y; }
-      if (hi) { acc[0][1].x += cur.x * s1.x; acc[0][1].y += cur.x * s1.y; }
-    } else {
-      if (lo) cmac(acc[0][0], cur, s0);
-      if (hi) cmac(acc[0][1], cur, s1);
-    }
-  };
-  bool any = false;
-  for (;;) {
-    const uint32_t g = min(gq, ge);   // uniform over the warp
-    if (g == kEnd) break;
-    const C c = coefS[g];
-    if (!any) {
-      cur = c;
-      any = true;
-    } else if (!same(c, cur)) {
-      flush();
-      s0 = s1 = czero<C>();
-      cur = c;
-    }
-    // the group's first T_up rows load while its T_dn slots are gathered
-    constexpr int NB = 4;
-    C v[NB][2];
-    double sg[NB];
-    int nb = 0;
-#pragma unroll
-    for (int i = 0; i < NB; ++i) {
-      if (nb == i && e + i < ne) {
-        const uint2 m = lst[e + i];
-        if ((m.y & 0xFFu) == g) {
-          ldcg_pair<C, false, false>(x + m.x, pcl, dim_dn, v[i][0], v[i][1]);
-          sg[i] = (m.y >> 31) ? -1.0 : 1.0;
-          nb = i + 1;
-        }
-      }
-    }
-    while (gq == g) {
-      const uint32_t w = word;
-      ++q;
-      if (q < q1) { word = __ldg(ellp + (size_t)q * 32); gq = __ldg(sd.dn_slot_grp + q); }
-      else gq = kEnd;
-      uint32_t o0, o1;
-      double g0, g1;
-      TIO::unpack<double>(w, o0, o1, g0, g1);
-      C a0[1], a1[1];
-      TIO::load_off(tile, o0, a0);
-      TIO::load_off(tile, o1, a1);
-      if (lo) cax(s0, g0, a0[0]);
-      if (hi) cax(s1, g1, a1[0]);
-    }
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-      if (i < nb) {
-        if (lo) cax(s0, sg[i], v[i][0]);
-        if (hi) cax(s1, sg[i], v[i][1]);
-      }
-    e += nb;
-    while (e < ne && (lst[e].y & 0xFFu) == g) {
-      C u0, u1;
-      ldcg_pair<C, false, false>(x + lst[e].x, pcl, dim_dn, u0, u1);
-      const double s = (lst[e].y >> 31) ? -1.0 : 1.0;
-      if (lo) cax(s0, s, u0);
-      if (hi) cax(s1, s, u1);
-      ++e;
-    }
-    ge = e < ne ? lst[e].y & 0xFFu : kEnd;
-  }
-  if (any) flush();
+  off_diagonal_c128(sd, tile, t, pcl, x, deg[0], [lst](int e) { return lst[e]; }, coefS, lo, hi,
+                    acc[0]);
 }
 
 // The a-posteriori check of step j (as k_conv_check), by one warp.
