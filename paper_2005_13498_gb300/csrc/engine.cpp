@@ -166,8 +166,12 @@ std::string tune_apply(const ApplyTuneTarget& t, cudaStream_t s, LaunchShape* sh
   }
   int64_t elems = 0;
   for (size_t i = 0; i < t.dim_up.size(); ++i) elems += (int64_t)t.dim_up[i] * t.dim_dn[i];
-  if (cands.size() == 1 || elems < (1 << 20)) {   // small problems: the default
+  if (cands.size() == 1 || elems < (1 << 20)) {   // small problems: a rule on the rows
+    int64_t rows = 0;
+    for (int d : t.dim_up) rows += d;
     *shape = cands.front();
+    for (const LaunchShape& c : cands)
+      if (c.cfg == apply_small_config(t.fp64, rows)) *shape = c;
     build(*shape);
     std::lock_guard<std::mutex> lock(mu);
     cache[key] = shape->cfg;

@@ -1933,6 +1933,22 @@ std::vector<LaunchShape> apply_candidates(int max_dim_up, int max_dim_dn, bool f
   return out;
 }
 
+// One row per CTA while the rows fit two CTAs on each of the 152 SMs, then
+// the entries that hold more CTAs per SM: complex64 two rows per CTA, three
+// CTAs (912 rows in a wave) or four.  us per product of one vector, and of
+// three where marked, entries 0 / 1 / 2 / 3 in complex64 and 4 / 5 / 6 / 24 in
+// complex128:
+//    70 x 70    8.3 /  6.8 /  8.2 /  6.2    16.5 / 12.4 / 10.3 / 11.3
+//   210 x 210   9.3 /  8.2 /  8.2 /  6.2    18.5 / 13.4 / 12.3 / 12.4
+//   364 x 91   10.3 /  8.2 /  8.2 /  8.3    24.6 / 11.1 / 14.4 / 10.3
+//   462 x 330  10.3 /  8.3 /  8.3 / 10.3    36.0 / 24.7 / 26.7 / 24.6
+//   792 x 66   20.5 / 20.6 / 18.5 / 28.7     152 / 55.4 / 79.9 / 59.5  (three)
+//   924 x 924  20.5 / 22.6 / 20.6 / 26.7     211 /  156 /  151 /  153
+int apply_small_config(bool fp64, int64_t rows) {
+  if (fp64) return rows <= 304 ? 6 : 24;
+  return rows <= 304 ? 3 : rows <= 912 ? 1 : 2;
+}
+
 LaunchShape apply_shape(int max_dim_up, int max_dim_dn, bool fp64, int n_groups) {
   std::vector<LaunchShape> c = apply_candidates(max_dim_up, max_dim_dn, fp64, n_groups);
   if (c.empty()) {
