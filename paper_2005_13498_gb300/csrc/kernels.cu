@@ -119,15 +119,16 @@ __device__ __forceinline__ void tma_bulk_g2s(void* dst, const void* src, uint32_
 // the last of them the pair index is clamped to the last pair of the row
 // (those sums are never stored).
 //  * complex64: no group sums.  Each entry reads its signed coefficient
-//    s c_g from the CTA's table coefQ[cs] = (s Re c, s Re c, s Im c, s Im c)
-//    (cs = 1 + 2 g + [s < 0]), one broadcast load, and accumulates
-//    a += (Re, Re) v, b += (Im, Im) v with two packed FMAs and no operand
-//    swaps; the row ends with acc += (a.x - b.y, a.y + b.x).
+//    s c_g from the CTA's table coefQ[cs] = (s Re c, s Im c)
+//    (cs = 1 + 2 g + [s < 0]), one broadcast load of 8 bytes (16 bytes with
+//    both parts doubled took a second wavefront of the L1 data pipe), and
+//    accumulates a += (Re, Re) v, b += (Im, Im) v with two packed FMAs and no
+//    operand swaps; the row ends with acc += (a.x - b.y, a.y + b.x).
 //  * complex128 (FP64-pipe bound): signed sums per bond group, multiplied
 //    by c_g once per group.
 template <int NB, int KA, bool VEC>
 __device__ __forceinline__ void tup_batch_c64(const float2* xrow, const int (&pk)[KA],
-                                              const float4* coefQ, int dim_dn,
+                                              const float2* coefQ, int dim_dn,
                                               const uint32_t (&css)[4], const uint32_t (&rows)[4],
                                               float2 (&sa)[2 * KA], float2 (&sb)[2 * KA],
                                               int nb = NB) {
@@ -154,11 +155,11 @@ __device__ __forceinline__ void tup_batch_c64(const float2* xrow, const int (&pk
 #pragma unroll
   for (int qq = 0; qq < NB; ++qq) {
     if (qq >= nb) continue;
-    const float4 q = coefQ[css[qq]];
+    const float2 c = coefQ[css[qq]];
 #pragma unroll
     for (int k = 0; k < 2 * KA; ++k) {
-      sa[k] = ffma2(make_float2(q.x, q.y), v[qq][k], sa[k]);
-      sb[k] = ffma2(make_float2(q.z, q.w), v[qq][k], sb[k]);
+      sa[k] = ffma2(make_float2(c.x, c.x), v[qq][k], sa[k]);
+      sb[k] = ffma2(make_float2(c.y, c.y), v[qq][k], sb[k]);
     }
   }
 }
@@ -166,7 +167,7 @@ __device__ __forceinline__ void tup_batch_c64(const float2* xrow, const int (&pk
 template <int NR, int PP, int KA, bool VEC, int NT>
 __device__ __forceinline__ void tup_chunk_c64(const SectorDev& sd,
                                               const float2* const (&xr)[NR],
-                                              const float4* coefQ, const int (&urow)[NR],
+                                              const float2* coefQ, const int (&urow)[NR],
                                               int nrows, int pc,
                                               int npairs, int dim_dn, float2 (&acc)[NR][2 * PP]) {
   constexpr int T = NT;
@@ -299,7 +300,7 @@ __device__ __forceinline__ void tup_chunk_c128(const SectorDev& sd,
 
 template <typename R, int NR, int PP, int KA, bool VEC, int NT = kApplyThreads>
 __device__ __forceinline__ void tup_chunk(const SectorDev& sd, const typename C2T<R>::T* x,
-                                          const typename C2T<R>::T* coefS, const float4* coefQ,
+                                          const typename C2T<R>::T* coefS, const float2* coefQ,
                                           const int (&urow)[NR], int nrows, int pc, int npairs,
                                           int dim_dn,
                                           typename C2T<R>::T (&acc)[NR][2 * PP]) {
@@ -319,7 +320,7 @@ __device__ __forceinline__ void tup_chunk(const SectorDev& sd, const typename C2
 template <typename R, int NR, int PP, int KA, bool VEC, int NT>
 __device__ __forceinline__ void tup_chunk_mv(const SectorDev& sd,
                                              const typename C2T<R>::T* const (&xr)[NR],
-                                             const typename C2T<R>::T* coefS, const float4* coefQ,
+                                             const typename C2T<R>::T* coefS, const float2* coefQ,
                                              int u, int nrows, int pc, int npairs, int dim_dn,
                                              typename C2T<R>::T (&acc)[NR][2 * PP]) {
   int urow[NR];
@@ -348,11 +349,11 @@ __device__ __forceinline__ void apply_dot_result(LanczosState* st, double* out_e
 
 // Shared-memory bytes in front of the TMA ring / end of the apply's dynamic
 // shared memory: the tile, the group coefficients, and for complex64 the
-// signed coefficient quads of the T_up gathers (16-byte aligned).
+// signed coefficients of the T_up gathers (16-byte aligned).
 __host__ __device__ inline size_t apply_coef_end(int max_dim_dn, int nr, int n_groups, bool fp64) {
   const size_t csz = fp64 ? sizeof(double2) : sizeof(float2);
   size_t off = ((size_t)(max_dim_dn + kZeroCols) * nr + (size_t)n_groups) * csz;
-  if (!fp64) off = ((off + 15) & ~(size_t)15) + (size_t)(1 + 2 * n_groups) * sizeof(float4);
+  if (!fp64) off = ((off + 15) & ~(size_t)15) + (size_t)(1 + 2 * n_groups) * sizeof(float2);
   return off;
 }
 
@@ -432,8 +433,8 @@ k_apply(BatchArgs a, int j) {
 
   C* tile = reinterpret_cast<C*>(smem_raw);              // [max_dim_dn + kZeroCols][NR]
   C* coefS = tile + (size_t)(a.max_dim_dn + kZeroCols) * NR;   // [n_groups]
-  // complex64: signed coefficient quads of the T_up gathers, [1 + 2 n_groups]
-  float4* coefQ = reinterpret_cast<float4*>(
+  // complex64: signed coefficients of the T_up gathers, [1 + 2 n_groups]
+  float2* coefQ = reinterpret_cast<float2*>(
       smem_raw + ((((size_t)(a.max_dim_dn + kZeroCols) * NR + (size_t)a.n_groups) * sizeof(C) + 15) &
                   ~(size_t)15));
   // TMA configurations: ring of S row chunks (128-byte aligned after
@@ -465,11 +466,11 @@ k_apply(BatchArgs a, int j) {
   for (int g = tid; g < a.n_groups; g += T) coefS[g] = reinterpret_cast<const C*>(cbase)[g];
   if constexpr (sizeof(R) == 4) {
     for (int i = tid; i <= 2 * a.n_groups; i += T) {
-      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+      float2 q = make_float2(0.f, 0.f);
       if (i > 0) {
         const float2 c = reinterpret_cast<const float2*>(cbase)[(i - 1) >> 1];
         const float sg = ((i - 1) & 1) ? -1.f : 1.f;
-        q = make_float4(sg * c.x, sg * c.x, sg * c.y, sg * c.y);
+        q = make_float2(sg * c.x, sg * c.y);
       }
       coefQ[i] = q;
     }
@@ -818,8 +819,23 @@ k_apply(BatchArgs a, int j) {
         const R de0 = sd.dn_eps ? (R)__ldg(sd.dn_eps + d0) : (R)0;
         const R de1 = (sd.dn_eps && has1) ? (R)__ldg(sd.dn_eps + d0 + 1) : (R)0;
         C xa[NR], xb[NR];
-        TIO::load(tile, d0, xa);
-        TIO::load(tile, d0 + 1, xb);    // zero column past the end
+        // (column d0 + 1 past the end: a zero column.)  Lanes read columns
+        // 2 l and 2 l + 1; with 16-byte columns lanes l and l + 4 of a quarter
+        // warp would meet in one bank group, so the upper half of each eight
+        // takes its two columns in the other order
+        const bool sw = TIO::kBytes == 16 && (lane & 4);
+        TIO::load(tile, d0 + (sw ? 1 : 0), xa);
+        TIO::load(tile, d0 + (sw ? 0 : 1), xb);
+        if constexpr (TIO::kBytes == 16) {
+#pragma unroll
+          for (int r = 0; r < NR; ++r) {
+            const C ya = xa[r], yb = xb[r];
+            xa[r].x = sw ? yb.x : ya.x;
+            xa[r].y = sw ? yb.y : ya.y;
+            xb[r].x = sw ? ya.x : yb.x;
+            xb[r].y = sw ? ya.y : yb.y;
+          }
+        }
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
           if (r < nrows) {
@@ -911,10 +927,10 @@ k_apply_tup(BatchArgs a, int j) {
 #pragma unroll
   for (int r = 0; r < NR; ++r) urow[r] = r < nrows ? ab.row[r] : ab.row[0];
 
-  // the group coefficients and (complex64) their signed quads, laid out as
+  // the group coefficients and (complex64) their signed copies, laid out as
   // in k_apply with an empty tile
   C* coefS = reinterpret_cast<C*>(smem_raw);
-  float4* coefQ = reinterpret_cast<float4*>(
+  float2* coefQ = reinterpret_cast<float2*>(
       smem_raw + (((size_t)a.n_groups * sizeof(C) + 15) & ~(size_t)15));
   const void* cbase;
   if (j >= 1) cbase = static_cast<const char*>(a.coefs) + (size_t)st->step * a.n_groups * sizeof(C);
@@ -923,11 +939,11 @@ k_apply_tup(BatchArgs a, int j) {
   for (int g = tid; g < a.n_groups; g += T) coefS[g] = reinterpret_cast<const C*>(cbase)[g];
   if constexpr (sizeof(R) == 4) {
     for (int i = tid; i <= 2 * a.n_groups; i += T) {
-      float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+      float2 q = make_float2(0.f, 0.f);
       if (i > 0) {
         const float2 c = reinterpret_cast<const float2*>(cbase)[(i - 1) >> 1];
         const float sg = ((i - 1) & 1) ? -1.f : 1.f;
-        q = make_float4(sg * c.x, sg * c.x, sg * c.y, sg * c.y);
+        q = make_float2(sg * c.x, sg * c.y);
       }
       coefQ[i] = q;
     }
