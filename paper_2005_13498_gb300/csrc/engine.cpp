@@ -607,7 +607,14 @@ std::string Engine::run(int n_steps, bool profile, double* kernel_ms, int64_t* l
     k.prof = static_cast<uint64_t*>(prof.p);
     for (int n = 0; n == 0 || n < n_steps; n += kKrylovSteps) {
       k.n_steps = std::min(kKrylovSteps, n_steps - n);
-      ED_TRY(launch_krylov(f, kry_vec_, k, kry_grid_, kry_smem_, s));
+      const cudaError_t e = launch_krylov(f, kry_vec_, k, kry_grid_, kry_smem_, s);
+      if (e == cudaErrorCooperativeLaunchTooLarge && n == 0) {
+        // fewer SMs at hand than the device has (a partitioned context)
+        cudaGetLastError();
+        kry_grid_ = 0;
+        return run(n_steps, profile, kernel_ms, launches, s);
+      }
+      ED_TRY(e);
     }
     if (profile) {
       uint64_t h[2 * KK_COUNT];
