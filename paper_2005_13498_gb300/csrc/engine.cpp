@@ -34,7 +34,8 @@ Engine::~Engine() {
   if (graph_) cudaGraphDestroy(graph_);
   for (cudaEvent_t e : ev_fork_) cudaEventDestroy(e);
   for (cudaEvent_t e : ev_check_) cudaEventDestroy(e);
-  if (side_) cudaStreamDestroy(side_);
+  for (cudaStream_t st : {side_, body_, body_side_})
+    if (st) cudaStreamDestroy(st);
 }
 
 size_t Engine::device_bytes() const {
@@ -246,6 +247,8 @@ std::string Engine::setup(const EngineConfig& cfg, const std::vector<SectorDev>&
   const int m = cfg.m;
   if (cfg.eps_tol > 0.0 && !side_) {
     ED_TRY(cudaStreamCreateWithFlags(&side_, cudaStreamNonBlocking));
+    ED_TRY(cudaStreamCreateWithFlags(&body_, cudaStreamNonBlocking));
+    ED_TRY(cudaStreamCreateWithFlags(&body_side_, cudaStreamNonBlocking));
     ev_fork_.assign(kMaxKrylov + 1, nullptr);
     ev_check_.assign(kMaxKrylov + 1, nullptr);
     for (int i = 0; i <= kMaxKrylov; ++i) {
@@ -515,41 +518,97 @@ std::string Engine::begin(const std::vector<double>& coefs, const std::vector<do
   return "";
 }
 
-std::string Engine::launch_step(cudaStream_t s, bool profile, cudaEvent_t* ev, int* kind_of,
-                                int* nev) {
-  const bool f = cfg_.fp64;
-  auto mark = [&](int kind) -> std::string {
-    if (!profile) return "";
+// Passes of the step graph that always run in the adaptive mode; the others
+// are the body of a conditional node.  Returning at once, each of them costs
+// its launch: with m = 30 and an exit after 7 or 8 vectors the skipped passes
+// took 0.14 of 3.09 ms per step of the Ns = 14 ladder.  A step that needs the
+// body waits for the check of pass kGatePass first (about 15 us).
+constexpr int kGatePass = 10;
+
+namespace {
+// Records around a launch in profile mode, then the launch.
+struct Marks {
+  bool on;
+  cudaEvent_t* ev;
+  int* kind_of;
+  int* nev;
+  std::string mark(int kind, cudaStream_t s) {
+    if (!on) return "";
     ED_TRY(cudaEventRecord(ev[*nev], s));
     kind_of[*nev] = kind;
     ++*nev;
     return "";
-  };
-  std::string err;
-#define STEP_LAUNCH(kind, call)                         \
-  do {                                                  \
-    if (!(err = mark(-1)).empty()) return err;          \
-    ED_TRY(call);                                       \
-    if (!(err = mark(kind)).empty()) return err;        \
+  }
+};
+}  // namespace
+#define STEP_LAUNCH(kind, call)                            \
+  do {                                                     \
+    if (!(err = mk.mark(-1, s)).empty()) return err;       \
+    ED_TRY(call);                                          \
+    if (!(err = mk.mark(kind, s)).empty()) return err;     \
   } while (0)
+
+std::string Engine::launch_passes(cudaStream_t s, cudaStream_t side, int j0, int j1, bool profile,
+                                  cudaEvent_t* ev, int* kind_of, int* nev) {
+  const bool f = cfg_.fp64;
+  Marks mk{profile, ev, kind_of, nev};
+  std::string err;
   // With the adaptive exit, the check of step j runs on the side stream
   // while pass j + 1 proceeds on s; pass j + 2 waits for it (a converged
   // check makes the later passes return at once, see lanczos_done).
   const bool adaptive = cfg_.eps_tol > 0.0;
-  for (int j = 1; j <= cfg_.m; ++j) {
-    if (adaptive && j >= 3) ED_TRY(cudaStreamWaitEvent(s, ev_check_[j - 2], 0));
+  for (int j = j0; j <= j1; ++j) {
+    if (adaptive && j - 2 >= j0) ED_TRY(cudaStreamWaitEvent(s, ev_check_[j - 2], 0));
     STEP_LAUNCH(KK_APPLY, launch_apply(f, args_, n_apply_, shape_, j, s));
     if (j < cfg_.m) {
       STEP_LAUNCH(KK_UPDATE, launch_update(f, args_, n_ew_, j, s));
       if (adaptive) {
         ED_TRY(cudaEventRecord(ev_fork_[j], s));
-        ED_TRY(cudaStreamWaitEvent(side_, ev_fork_[j], 0));
-        ED_TRY(launch_conv_check(args_, j, side_));
-        ED_TRY(cudaEventRecord(ev_check_[j], side_));
+        ED_TRY(cudaStreamWaitEvent(side, ev_fork_[j], 0));
+        ED_TRY(launch_conv_check(args_, j, side));
+        ED_TRY(cudaEventRecord(ev_check_[j], side));
       }
     }
   }
-  if (adaptive && cfg_.m >= 2) ED_TRY(cudaStreamWaitEvent(s, ev_check_[cfg_.m - 1], 0));
+  const int last = std::min(j1, cfg_.m - 1);   // the last check made here
+  if (adaptive && last >= j0) ED_TRY(cudaStreamWaitEvent(s, ev_check_[last], 0));
+  return "";
+}
+
+std::string Engine::launch_step(cudaStream_t s, bool profile, cudaEvent_t* ev, int* kind_of,
+                                int* nev) {
+  const bool f = cfg_.fp64;
+  Marks mk{profile, ev, kind_of, nev};
+  std::string err;
+  const bool gated = cfg_.eps_tol > 0.0 && !profile && cfg_.m > kGatePass + 2;
+  err = launch_passes(s, side_, 1, gated ? kGatePass : cfg_.m, profile, ev, kind_of, nev);
+  if (!err.empty()) return err;
+  if (gated) {   // s is being captured (capture())
+    cudaStreamCaptureStatus status;
+    cudaGraph_t graph = nullptr;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t ndeps = 0;
+    ED_TRY(cudaStreamGetCaptureInfo(s, &status, nullptr, &graph, nullptr, nullptr, nullptr));
+    if (status != cudaStreamCaptureStatusActive) return "step graph: the stream is not being captured";
+    cudaGraphConditionalHandle handle;
+    ED_TRY(cudaGraphConditionalHandleCreate(&handle, graph, 0, cudaGraphCondAssignDefault));
+    ED_TRY(launch_gate(args_, handle, s));
+    ED_TRY(cudaStreamGetCaptureInfo(s, &status, nullptr, &graph, &deps, nullptr, &ndeps));
+    cudaGraphNodeParams p = {};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = handle;
+    p.conditional.type = cudaGraphCondTypeIf;
+    p.conditional.size = 1;
+    cudaGraphNode_t node;
+    ED_TRY(cudaGraphAddNode(&node, graph, deps, nullptr, ndeps, &p));
+    ED_TRY(cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
+    ED_TRY(cudaStreamBeginCaptureToGraph(body_, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                         cudaStreamCaptureModeThreadLocal));
+    err = launch_passes(body_, body_side_, kGatePass + 1, cfg_.m, false, nullptr, nullptr, nullptr);
+    const cudaError_t e = cudaStreamEndCapture(body_, nullptr);
+    if (!err.empty()) return err;
+    ED_TRY(e);
+  }
   STEP_LAUNCH(KK_EXPM, launch_expm(args_, s));
   STEP_LAUNCH(KK_COMBINE, launch_combine(f, args_, n_ew_, s));
   if (cfg_.energy) STEP_LAUNCH(KK_ENERGY, launch_apply(f, args_, n_apply_, shape_, -1, s));
@@ -557,9 +616,9 @@ std::string Engine::launch_step(cudaStream_t s, bool profile, cudaEvent_t* ev, i
     if (need_psiT_) STEP_LAUNCH(KK_OVERLAP, launch_psiT(s));
     STEP_LAUNCH(KK_OVERLAP, launch_overlap(f, args_, oargs_, n_ew_, s));
   }
-#undef STEP_LAUNCH
   return "";
 }
+#undef STEP_LAUNCH
 
 cudaError_t Engine::launch_psiT(cudaStream_t s) {
   const SectorDev& sp = sectors_[vecs_[oargs_.psi_index].sector];

@@ -131,9 +131,14 @@ class Engine {
   double U_ = 0.0, break_tol_ = 0.0, tau_ = 0.0;
   int n_apply_ = 0, n_ew_ = 0;
   LaunchShape shape_{};
+  // Lanczos passes j0 .. j1 on s, with the adaptive checks on `side`
+  std::string launch_passes(cudaStream_t s, cudaStream_t side, int j0, int j1, bool profile,
+                            cudaEvent_t* ev, int* kind_of, int* nev);
   // adaptive exit: side stream for the convergence checks and the events
-  // that fork check j after update j and join it before pass j + 2
-  cudaStream_t side_ = nullptr;
+  // that fork check j after update j and join it before pass j + 2; in the
+  // step graph the passes after kGatePass are the body of a conditional node,
+  // captured on body_ with the checks on body_side_
+  cudaStream_t side_ = nullptr, body_ = nullptr, body_side_ = nullptr;
   std::vector<cudaEvent_t> ev_fork_, ev_check_;
   BatchArgs args_{};
   OverlapArgs oargs_{};

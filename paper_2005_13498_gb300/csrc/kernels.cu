@@ -1408,6 +1408,13 @@ __global__ void __launch_bounds__(32) k_conv_check(BatchArgs a, int j) {
   }
 }
 
+__global__ void __launch_bounds__(32) k_gate(BatchArgs a, cudaGraphConditionalHandle h) {
+  bool more = false;
+  for (int v = threadIdx.x; v < a.nvec; v += 32) more = more || !(a.st[v].stopped || a.st[v].conv_m > 0);
+  more = __any_sync(0xffffffffu, more);
+  if (threadIdx.x == 0) cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
 // ------------------------------------------------------ combine / observe
 // psi <- sum_j comb_j x_j (in place over x_1), fused with |psi|^2 and
 // sum_k w_d[k] |psi_k|^2 (Sec. 3.5), then the per-step bookkeeping.
@@ -2086,6 +2093,11 @@ cudaError_t launch_update(bool fp64, const BatchArgs& a, int nblk, int j, cudaSt
 
 cudaError_t launch_conv_check(const BatchArgs& a, int j, cudaStream_t s) {
   k_conv_check<<<a.nvec, 32, 0, s>>>(a, j);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gate(const BatchArgs& a, cudaGraphConditionalHandle h, cudaStream_t s) {
+  k_gate<<<1, 32, 0, s>>>(a, h);
   return cudaGetLastError();
 }
 

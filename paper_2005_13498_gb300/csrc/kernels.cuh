@@ -142,6 +142,9 @@ cudaError_t launch_apply(bool fp64, const BatchArgs& a, int n_apply_blocks,
                          const LaunchShape& sh, int j, cudaStream_t s);
 cudaError_t launch_update(bool fp64, const BatchArgs& a, int n_ew_blocks, int j,
                           cudaStream_t s);
+// Sets a graph's conditional handle to whether any vector still needs Lanczos
+// passes (the checks of the passes so far have finished).
+cudaError_t launch_gate(const BatchArgs& a, cudaGraphConditionalHandle h, cudaStream_t s);
 cudaError_t launch_expm(const BatchArgs& a, cudaStream_t s);
 // y[b] = exp(-i tau T_b) e_1 for batch real symmetric tridiagonals T_b of
 // order n <= kMaxKrylov (alpha: batch x n, beta: batch x (n - 1), y: batch x n
