@@ -34,7 +34,10 @@ inline DoccShape docc_shape(int dim_up, int dim_dn) {
   s.threads = dim_dn >= kDoccThreads ? kDoccThreads : (dim_dn + 31) / 32 * 32;
   s.cols = (dim_dn + s.threads - 1) / s.threads;
   const int chunks = kDoccBlocks / s.cols;   // >= 20 (rows have at most 12870 columns)
-  s.rows = (dim_up + chunks - 1) / chunks;
+  // at least 16 rows a thread: folding its sums costs as much as about 9 rows
+  // (us per call with at least 1 / 8 / 16: 495 x 495 90 / 57 / 60, 70 x 70 49 /
+  // 50 / 46, 924 x 924 92 / 82 / 73)
+  s.rows = std::max(16, (dim_up + chunks - 1) / chunks);
   s.blocks = s.cols * ((dim_up + s.rows - 1) / s.rows);
   return s;
 }
