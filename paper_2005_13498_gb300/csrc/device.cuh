@@ -308,7 +308,8 @@ __device__ __forceinline__ bool same(double a, double b) {
 // A = 0), and a real coefficient costs half a complex product.  On the 2x7
 // ladder that is 75 operations per element where sums and products per group
 // and direction took 104: Lanczos pass 1.95 -> 1.55 ms (90 % of the pipe), the
-// step 65.6 -> 52.2 ms with the update.  With the T_up additions and the
+// step 65.6 -> 52.2 ms with the update; 1.51 and 51.0 ms with the Lanczos scale
+// in the caller's coefficients.  With the T_up additions and the
 // products selected by short conditional blocks the compiler predicated them,
 // and switched-off instructions take the pipe's time as well: 1.94 ms.
 // lo, hi: which of the lane's two columns to compute

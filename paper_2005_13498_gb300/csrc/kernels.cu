@@ -463,7 +463,15 @@ k_apply(BatchArgs a, int j) {
   if (j >= 1) cbase = static_cast<const char*>(a.coefs) + (size_t)st->step * a.n_groups * sizeof(C);
   else if (j == 0) cbase = a.coefs;
   else cbase = static_cast<const char*>(a.coefs_obs) + (size_t)st->step * a.n_groups * sizeof(C);
-  for (int g = tid; g < a.n_groups; g += T) coefS[g] = reinterpret_cast<const C*>(cbase)[g];
+  // LEAN: the Lanczos scale s_j goes into the coefficients and the diagonal's
+  // table instead of two products per element (2x7 ladder: pass 1.55 -> 1.51 ms;
+  // rms error of a product against 80 bits 3.05e-16 -> 3.02e-16)
+  const R s_coef = LEAN && j >= 1 ? (R)st->inv_scale[j] : (R)1;
+  for (int g = tid; g < a.n_groups; g += T) {
+    C c = reinterpret_cast<const C*>(cbase)[g];
+    if constexpr (LEAN) { c.x *= s_coef; c.y *= s_coef; }
+    coefS[g] = c;
+  }
   if constexpr (sizeof(R) == 4) {
     for (int i = tid; i <= 2 * a.n_groups; i += T) {
       float2 q = make_float2(0.f, 0.f);
@@ -524,7 +532,7 @@ k_apply(BatchArgs a, int j) {
   if constexpr (LEAN) {
     ue0 = __ldg(sd.up_off + urow[0]);
     une = __ldg(sd.up_off + urow[0] + 1) - ue0;
-    if (tid <= kMaxSites) utab[LEAN ? tid : 0] = (R)a.U * (R)tid;
+    if (tid <= kMaxSites) utab[LEAN ? tid : 0] = s_coef * ((R)a.U * (R)tid);
     for (int i = tid; i < min(une, kLean); i += T) {
       const uint32_t en = __ldg(sd.up_ent + ue0 + i);
       upl[i] = make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
@@ -843,7 +851,7 @@ k_apply(BatchArgs a, int j) {
             if constexpr (LEAN) {   // no conversions and products on the FP64 pipe
               g0 = utab[__popc(uw[r] & dw0)];
               g1 = utab[__popc(uw[r] & dw1)];
-              if (sd.up_eps) { g0 += eu[r] + de0; g1 += eu[r] + de1; }
+              if (sd.up_eps) { g0 += s_coef * (eu[r] + de0); g1 += s_coef * (eu[r] + de1); }
             } else {
               g0 = U * (R)__popc(uw[r] & dw0) + eu[r] + de0;
               g1 = U * (R)__popc(uw[r] & dw1) + eu[r] + de1;
@@ -854,10 +862,17 @@ k_apply(BatchArgs a, int j) {
             a1.x += g1 * xb[r].x;
             a1.y += g1 * xb[r].y;
             C o0, o1;
-            o0.x = sinr[r] * a0.x - sprevr[r] * pv[r][2 * k].x;
-            o0.y = sinr[r] * a0.y - sprevr[r] * pv[r][2 * k].y;
-            o1.x = sinr[r] * a1.x - sprevr[r] * pv[r][2 * k + 1].x;
-            o1.y = sinr[r] * a1.y - sprevr[r] * pv[r][2 * k + 1].y;
+            if constexpr (LEAN) {
+              o0.x = a0.x - sprevr[r] * pv[r][2 * k].x;
+              o0.y = a0.y - sprevr[r] * pv[r][2 * k].y;
+              o1.x = a1.x - sprevr[r] * pv[r][2 * k + 1].x;
+              o1.y = a1.y - sprevr[r] * pv[r][2 * k + 1].y;
+            } else {
+              o0.x = sinr[r] * a0.x - sprevr[r] * pv[r][2 * k].x;
+              o0.y = sinr[r] * a0.y - sprevr[r] * pv[r][2 * k].y;
+              o1.x = sinr[r] * a1.x - sprevr[r] * pv[r][2 * k + 1].x;
+              o1.y = sinr[r] * a1.y - sprevr[r] * pv[r][2 * k + 1].y;
+            }
             if (!rdone[r]) store_pair<C, VEC, true>(wr[r] + (size_t)urow[r] * dim_dn, p, dim_dn, o0, o1);
             const R dre = xa[r].x * o0.x + xa[r].y * o0.y + xb[r].x * o1.x + xb[r].y * o1.y;
             if constexpr (MV) dacc_r[r] += dre;
