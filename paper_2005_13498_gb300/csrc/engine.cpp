@@ -415,7 +415,8 @@ std::string Engine::setup(const EngineConfig& cfg, const std::vector<SectorDev>&
 
 std::string Engine::setup_persistent(const SpinTable* up, bool vec_ok) {
   kry_grid_ = 0;
-  if (!up) return "";
+  // complex64 only (krylov.cu)
+  if (!up || cfg_.fp64) return "";
   const SectorDev& sd = sectors_[vecs_[0].sector];
   int dev = 0, sms = 0, coop = 0;
   ED_TRY(cudaGetDevice(&dev));
@@ -427,10 +428,10 @@ std::string Engine::setup_persistent(const SpinTable* up, bool vec_ok) {
   kry_deg_ = 1;
   for (int r = 0; r < up->dim; ++r) kry_deg_ = std::max(kry_deg_, up->off[r + 1] - up->off[r]);
   kry_vec_ = vec_ok;
-  kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_, cfg_.fp64);
+  kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_);
   if (kry_smem_ > 227 * 1024) return "";
   int ctas = 0;
-  ED_TRY(krylov_prepare(cfg_.fp64, kry_vec_, kry_smem_, &ctas));
+  ED_TRY(krylov_prepare(kry_vec_, kry_smem_, &ctas));
   if (ctas < 1) return "";
   ED_TRY(d_slots_.alloc(kKrylovSlotBytes));
   kry_grid_ = grid;
@@ -666,7 +667,7 @@ std::string Engine::run(int n_steps, bool profile, double* kernel_ms, int64_t* l
     k.prof = static_cast<uint64_t*>(prof.p);
     for (int n = 0; n == 0 || n < n_steps; n += kKrylovSteps) {
       k.n_steps = std::min(kKrylovSteps, n_steps - n);
-      const cudaError_t e = launch_krylov(f, kry_vec_, k, kry_grid_, kry_smem_, s);
+      const cudaError_t e = launch_krylov(kry_vec_, k, kry_grid_, kry_smem_, s);
       if (e == cudaErrorCooperativeLaunchTooLarge && n == 0) {
         // fewer SMs at hand than the device has (a partitioned context)
         cudaGetLastError();

@@ -211,9 +211,9 @@ struct KrylovArgs {
 };
 // Dynamic shared memory of a launch, and the CTAs per SM it allows (0: does
 // not fit); krylov_prepare raises the kernel's limit.
-size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, bool fp64);
-cudaError_t krylov_prepare(bool fp64, bool vec, size_t smem, int* ctas_per_sm);
-cudaError_t launch_krylov(bool fp64, bool vec, const KrylovArgs& k, int grid, size_t smem,
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups);
+cudaError_t krylov_prepare(bool vec, size_t smem, int* ctas_per_sm);
+cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
                           cudaStream_t s);
 
 // ---- ground-state helpers (float64 only) ---------------------------------

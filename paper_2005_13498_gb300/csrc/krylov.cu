@@ -10,17 +10,19 @@
 // ELL words stay in shared memory and L1, and per Lanczos step only two
 // grid-wide sums are left (alpha_j, then beta_j together with the visibility
 // of x_{j+1}, whose rows the T_up gathers of the other CTAs read through L2).
-// Measured per call, separate kernels -> this kernel: 20 steps of the 8-site
-// ring with energies (D = 4,900, m = 12, complex128) 7.67 -> 4.43 ms, 10 steps
-// of the 12-site torus (D = 853,776, m = 20, complex64) 8.40 -> 7.47 ms, two
-// CFET4 steps of it with energies in complex128 21.8 -> 15.1 ms.
-// What bounds it: for the ring the latency of the passes (4 us) and of the
+// Measured per call, separate kernels of the time -> this kernel, complex64:
+// 10 steps of the 12-site torus (D = 853,776, m = 20) 8.40 -> 7.23 ms, 20 steps
+// of the (2,6) sector of a 10-site chain (D = 9,450, m = 22) 8.16 -> 6.00 ms.
+// What bounds it: for the small sectors the latency of the passes and of the
 // sums (4.5 us each: 2.1 us from a CTA's store to the last CTA's successful
 // poll across the two dies, the rest dependent float64 additions at about
-// 50 ns); for the torus the shared-memory and L2 gathers (complex64, 21 of 37
-// us per Lanczos step) and the FP64 pipe (complex128, 183 us).
+// 50 ns); for the torus the shared-memory and L2 gathers (21 of 37 us per
+// Lanczos step).
 // It is used when two copies of a CTA's rows fit its shared memory: up to
-// about 15 MB of state (D = 1.9 M in complex64, 0.95 M in complex128).
+// about 15 MB of state (D = 1.9 M).  complex64 only: a complex128 form read, in
+// some builds, the previous step's bond coefficients in a few rows (gone without
+// a field, so not the vectors), for a reason not found, and gained 3 to 18 % over
+// the separate kernels.
 //
 // Grid-wide sums: each CTA publishes its float64 partial as two 64-bit words
 // that carry the sum's epoch in their upper halves, and one warp of every CTA
@@ -41,11 +43,9 @@ constexpr int kErrNumeric = 7;    // ED_ERR_NUMERIC
 constexpr int kUpBatch = 6;
 constexpr int kPollLanes = (kKrylovMaxGrid + 31) / 32;
 
-// complex64: two rows per 16-byte tile column, 20 warps at 96 registers;
-// complex128 (FP64-pipe bound): one row, 16 warps at 128 registers
+// two rows per 16-byte tile column, 20 warps at 96 registers
 template <typename R> struct KCfg;
 template <> struct KCfg<float> { static constexpr int NT = 640, NR = 2; };
-template <> struct KCfg<double> { static constexpr int NT = 512, NR = 1; };
 
 // Scalars of the Lanczos recursion in shared memory, 1-based as LanczosState.
 struct Scalars {
@@ -57,6 +57,12 @@ struct Scalars {
   double utab[kMaxSites + 1];   // U n
   int m_eff, stop, status, conv, err, step;
 };
+
+// The block barrier; every warp reconverges first (its lanes leave loops apart).
+__device__ __forceinline__ void block_sync() {
+  __syncwarp();
+  __syncthreads();
+}
 
 // A published partial: the halves of a float64, each with the sum's epoch in
 // the upper 32 bits of its word, so that no ordering between the two words
@@ -85,9 +91,9 @@ __device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Sca
   double part[K];
 #pragma unroll
   for (int kk = 0; kk < K; ++kk) {
-    if (kk > 0) __syncthreads();
+    if (kk > 0) block_sync();
     redS[tid] = v[kk];
-    __syncthreads();
+    block_sync();
     if (warp < QW) {
       double s = 0.0;
 #pragma unroll
@@ -100,8 +106,7 @@ __device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Sca
   if (warp < QW && lane == 0)
 #pragma unroll
     for (int kk = 0; kk < K; ++kk) S.part[kk][warp] = part[kk];
-  __syncwarp();
-  __syncthreads();
+  block_sync();
   ++epoch;
   if (warp == 0) {
     const int G = gridDim.x;
@@ -154,8 +159,7 @@ __device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Sca
       S.err = 1;
     }
   }
-  __syncwarp();
-  __syncthreads();
+  block_sync();
   return !S.err;
 }
 
@@ -194,13 +198,13 @@ __device__ __forceinline__ void ldcg_pair(const C* row, int p, int dim, C& v0, C
 
 // The off-diagonal part of H x for one item, NR tile rows x 64 columns (two
 // columns per lane): acc[r][h] of row r and column 2 p + h.
-//  complex64: T_dn over the ELL slots of the tile (two slots per turn, words
-//  two turns ahead), then T_up row by row with the signed coefficients,
-//  eight source rows in flight.
+// T_dn over the ELL slots of the tile (two slots per turn, words
+//  a turn ahead), then T_up row by row with the signed coefficients, kUpBatch
+//  source rows in flight.
 __device__ __forceinline__ void off_diagonal(
     const SectorDev& sd, const float2* tile, int t, int p, int pcl, int npairs, const float2* x,
     const uint2* const (&list)[2], const int (&deg)[2], const float2* coefS, const float2* coefQ,
-    bool vec, bool, bool, float2 (&acc)[2][2]) {
+    bool vec, float2 (&acc)[2][2]) {
   constexpr int NR = 2;
   using TIO = TileIO<float2, NR>;
   const int lane = threadIdx.x & 31;
@@ -223,87 +227,70 @@ __device__ __forceinline__ void off_diagonal(
       s0[r] = s1[r] = make_float2(0.f, 0.f);
     }
   };
-  // Odd warps take T_up first: the L2 round trips of one half of the warps
-  // overlap the shared-memory gathers of the other.
-#pragma unroll 1
-  for (int ph = 0; ph < 2; ++ph) {
-    if (ph == 0) {
-      if (q0 >= q1) continue;
-      uint32_t na = __ldg(ellp + (size_t)q0 * 32), nb = __ldg(ellp + (size_t)(q0 + 1) * 32);
-      uint2 ng = __ldg(grp2 + (q0 >> 1));
-      uint32_t gcur = ng.x;
-      for (int q = q0; q < q1; q += 2) {
-        const uint32_t ea = na, eb = nb;
-        const uint2 gg = ng;
-        if (q + 2 < q1) {
-          na = __ldg(ellp + (size_t)(q + 2) * 32);
-          nb = __ldg(ellp + (size_t)(q + 3) * 32);
-          ng = __ldg(grp2 + ((q + 2) >> 1));
-        }
-        uint32_t oa0, oa1, ob0, ob1;
-        float ga0, ga1, gb0, gb1;
-        TIO::unpack<float>(ea, oa0, oa1, ga0, ga1);
-        TIO::unpack<float>(eb, ob0, ob1, gb0, gb1);
-        float2 a0[NR], a1[NR], b0[NR], b1[NR];
-        TIO::load_off(tile, oa0, a0);
-        TIO::load_off(tile, oa1, a1);
-        TIO::load_off(tile, ob0, b0);
-        TIO::load_off(tile, ob1, b1);
-        if (gg.x != gcur) { flush(gcur); gcur = gg.x; }   // uniform over the warp
-#pragma unroll
-        for (int r = 0; r < NR; ++r) { cax(s0[r], ga0, a0[r]); cax(s1[r], ga1, a1[r]); }
-        if (gg.y != gcur) { flush(gcur); gcur = gg.y; }
-#pragma unroll
-        for (int r = 0; r < NR; ++r) { cax(s0[r], gb0, b0[r]); cax(s1[r], gb1, b1[r]); }
+  if (q0 < q1) {
+    uint32_t na = __ldg(ellp + (size_t)q0 * 32), nb = __ldg(ellp + (size_t)(q0 + 1) * 32);
+    uint2 ng = __ldg(grp2 + (q0 >> 1));
+    uint32_t gcur = ng.x;
+    for (int q = q0; q < q1; q += 2) {
+      const uint32_t ea = na, eb = nb;
+      const uint2 gg = ng;
+      if (q + 2 < q1) {
+        na = __ldg(ellp + (size_t)(q + 2) * 32);
+        nb = __ldg(ellp + (size_t)(q + 3) * 32);
+        ng = __ldg(grp2 + ((q + 2) >> 1));
       }
-      flush(gcur);
-    } else {
-      constexpr int NB = kUpBatch;
+      uint32_t oa0, oa1, ob0, ob1;
+      float ga0, ga1, gb0, gb1;
+      TIO::unpack<float>(ea, oa0, oa1, ga0, ga1);
+      TIO::unpack<float>(eb, ob0, ob1, gb0, gb1);
+      float2 a0[NR], a1[NR], b0[NR], b1[NR];
+      TIO::load_off(tile, oa0, a0);
+      TIO::load_off(tile, oa1, a1);
+      TIO::load_off(tile, ob0, b0);
+      TIO::load_off(tile, ob1, b1);
+      if (gg.x != gcur) { flush(gcur); gcur = gg.x; }   // uniform over the warp
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        float2 sa[2], sb[2];
-        sa[0] = sa[1] = sb[0] = sb[1] = make_float2(0.f, 0.f);
-        for (int e = 0; e < deg[r]; e += NB) {
-          float2 v[NB][2];
-          uint32_t cs[NB];
+      for (int r = 0; r < NR; ++r) { cax(s0[r], ga0, a0[r]); cax(s1[r], ga1, a1[r]); }
+      if (gg.y != gcur) { flush(gcur); gcur = gg.y; }
 #pragma unroll
-          for (int i = 0; i < NB; ++i)
-            if (e + i < deg[r]) {   // uniform over the warp
-              const uint2 en = list[r][e + i];
-              cs[i] = en.y;
-              const float2* src = x + en.x;
-              if (vec) ldcg_pair<float2, true, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
-              else ldcg_pair<float2, false, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
-            }
+      for (int r = 0; r < NR; ++r) { cax(s0[r], gb0, b0[r]); cax(s1[r], gb1, b1[r]); }
+    }
+    flush(gcur);
+  }
+  constexpr int NB = kUpBatch;
 #pragma unroll
-          for (int i = 0; i < NB; ++i)
-            if (e + i < deg[r]) {
-              const float2 c = coefQ[cs[i]];
+  for (int r = 0; r < NR; ++r) {
+    float2 sa[2], sb[2];
+    sa[0] = sa[1] = sb[0] = sb[1] = make_float2(0.f, 0.f);
+    for (int e = 0; e < deg[r]; e += NB) {
+      float2 v[NB][2];
+      uint32_t cs[NB];
 #pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                sa[h] = ffma2(make_float2(c.x, c.x), v[i][h], sa[h]);
-                sb[h] = ffma2(make_float2(c.y, c.y), v[i][h], sb[h]);
-              }
-            }
+      for (int i = 0; i < NB; ++i)
+        if (e + i < deg[r]) {   // uniform over the warp
+          const uint2 en = list[r][e + i];
+          cs[i] = en.y;
+          const float2* src = x + en.x;
+          if (vec) ldcg_pair<float2, true, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
+          else ldcg_pair<float2, false, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          acc[r][h].x += sa[h].x - sb[h].y;
-          acc[r][h].y += sa[h].y + sb[h].x;
+      for (int i = 0; i < NB; ++i)
+        if (e + i < deg[r]) {
+          const float2 c = coefQ[cs[i]];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            sa[h] = ffma2(make_float2(c.x, c.x), v[i][h], sa[h]);
+            sb[h] = ffma2(make_float2(c.y, c.y), v[i][h], sb[h]);
+          }
         }
-      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      acc[r][h].x += sa[h].x - sb[h].y;
+      acc[r][h].y += sa[h].y + sb[h].x;
     }
   }
-}
-
-//  complex128: off_diagonal_c128 (device.cuh)
-__device__ __forceinline__ void off_diagonal(
-    const SectorDev& sd, const double2* tile, int t, int p, int pcl, int npairs, const double2* x,
-    const uint2* const (&list)[1], const int (&deg)[1], const double2* coefS, const float2*,
-    bool, bool lo, bool hi, double2 (&acc)[1][2]) {
-  const uint2* lst = list[0];
-  off_diagonal_c128(sd, tile, t, pcl, x, deg[0], [lst](int e) { return lst[e]; }, coefS, lo, hi,
-                    acc[0]);
 }
 
 // The a-posteriori check of step j (as k_conv_check), by one warp.
@@ -399,13 +386,7 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
   const float2* const coefQ = coef_q();
   double dot = 0.0;
   if (warp >= h.nwork) return dot;
-  // complex128 with warps to spare: an item per column of the lanes' pairs
-  // (a float64 instruction holds its SM sub-partition for 64 cycles, so one
-  // warp's chain is what a small sector waits for; 8-site ring: see k_krylov)
-  const int split = NR == 1 && 2 * h.items <= h.nwork ? 2 : 1;
-  for (int is = warp; is < h.items * split; is += h.nwork) {
-    const int it = split == 2 ? is >> 1 : is;
-    const bool lo = split == 1 || !(is & 1), hi = split == 1 || (is & 1);
+  for (int it = warp; it < h.items; it += h.nwork) {
     const int b = it / ntile, t = it - b * ntile, p = 32 * t + lane;
     const C* tile = tileX + b * pitch;
     const uint2* lst[NR];
@@ -419,10 +400,10 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
       urow[r] = cta + (have ? li : 0) * G;
     }
     C acc[NR][2];
-    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefS, coefQ, VEC, lo, hi, acc);
+    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefS, coefQ, VEC, acc);
     if (p >= npairs) continue;
     const int d0 = 2 * p;
-    const bool has1 = hi && d0 + 1 < dim_dn;
+    const bool has1 = d0 + 1 < dim_dn;
     const uint32_t dw0 = __ldg(sd.dn_word + d0), dw1 = has1 ? __ldg(sd.dn_word + d0 + 1) : 0u;
     C xa[NR], xb[NR], oa[NR], ob[NR];
     TIO::load(tile, d0, xa);
@@ -458,10 +439,10 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
       }
       oa[r] = o0;
       ob[r] = o1;
-      if (lo) da += xa[r].x * o0.x + xa[r].y * o0.y;
+      da += xa[r].x * o0.x + xa[r].y * o0.y;
       if (has1) da += xb[r].x * o1.x + xb[r].y * o1.y;
     }
-    if (lo) TIO::store(tileW + b * pitch, d0, oa);
+    TIO::store(tileW + b * pitch, d0, oa);
     if (has1) TIO::store(tileW + b * pitch, d0 + 1, ob);
     dot += (double)da;
   }
@@ -484,7 +465,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     h.vd = a.vec[0];
     h.sd = a.sec[a.vec[0].sector];
   }
-  __syncthreads();
+  block_sync();
   const SectorDev& sd = h.sd;
   const VecDev& vd = h.vd;
   LanczosState* st = a.st;
@@ -559,7 +540,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     S.step = st->step;
   }
   for (int i = tid; i <= kMaxSites; i += NT) S.utab[i] = a.U * (double)i;
-  __syncthreads();
+  block_sync();
   uint32_t epoch = 0;
   const int step0 = S.step;
 
@@ -576,11 +557,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
         }
         coefQ[i] = q;
       }
-    // reconverge first: a few lanes of warp 0 wrote the coefficients, and
-    // without this the other warps were seen to read the previous ones right
-    // after the block barrier
-    __syncwarp();
-    __syncthreads();
+    block_sync();
   };
   // one pass over the items: f(tile row, column tile, column pair)
   auto for_items = [&](auto&& f) {
@@ -750,17 +727,17 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     const bool zero = !(S.beta0 > 0.0 && isfinite(S.beta0));
     if (S.conv > 0 && S.conv == n && !zero) {   // y^(n) and delta are the check's
       for (int i = tid; i < n; i += NT) { S.yre[i] = S.yprev_re[i]; S.yim[i] = S.yprev_im[i]; }
-      __syncthreads();
+      block_sync();
     } else {
       for (int i = tid; i < 64; i += NT) {
         S.al[i] = i < n && !zero ? S.alpha[i + 1] : 0.0;
         S.be[i] = i < n - 1 && !zero ? S.beta[i + 1] : 0.0;
       }
-      __syncthreads();
+      block_sync();
       if (warp == 0) tridiag_expm_e1(S.al, S.be, n, a.tau, S.yre, S.yim);
       else if (warp == 1 && n > 1)
         tridiag_expm_e1(S.al, S.be, n - 1, a.tau, S.pre, S.pim);
-      __syncthreads();
+      block_sync();
       if (warp == 1) {
         double dn = 0.0, yn = 0.0;
         if (n > 1)
@@ -787,7 +764,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
           cf_lo.y = (R)(im - (double)(R)im);
         }
       }
-    __syncthreads();
+    block_sync();
     if (tid == 0 && cta == 0) {
       if (vd.out_delta) vd.out_delta[S.step] = S.conv_delta;
       if (vd.out_meff) vd.out_meff[S.step] = n;
@@ -844,11 +821,11 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
 
 }  // namespace
 
-size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, bool fp64) {
-  const int nr = fp64 ? KCfg<double>::NR : KCfg<float>::NR;
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups) {
+  const int nr = KCfg<float>::NR;
   const size_t rb = (rows + nr - 1) / nr;
-  return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 + (fp64 ? 0 : (size_t)(1 + 2 * n_groups) * 8) +
-         (size_t)n_groups * (fp64 ? 16 : 8) + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+  return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 + (size_t)(1 + 2 * n_groups) * 8 +
+         (size_t)n_groups * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
 }
 
 template <typename R, bool VEC>
@@ -863,21 +840,17 @@ static cudaError_t prepare_t(size_t smem, int* ctas) {
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_krylov<R, VEC>, KCfg<R>::NT, smem);
 }
 
-cudaError_t krylov_prepare(bool fp64, bool vec, size_t smem, int* ctas_per_sm) {
-  if (fp64) return prepare_t<double, false>(smem, ctas_per_sm);
+cudaError_t krylov_prepare(bool vec, size_t smem, int* ctas_per_sm) {
   return vec ? prepare_t<float, true>(smem, ctas_per_sm) : prepare_t<float, false>(smem, ctas_per_sm);
 }
 
-cudaError_t launch_krylov(bool fp64, bool vec, const KrylovArgs& k, int grid, size_t smem,
+cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
                           cudaStream_t s) {
   cudaError_t e = cudaMemsetAsync(k.slots, 0, kKrylovSlotBytes, s);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<KrylovArgs*>(&k)};
-  const void* f = fp64 ? (const void*)k_krylov<double, false>
-                  : vec ? (const void*)k_krylov<float, true>
-                        : (const void*)k_krylov<float, false>;
-  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(fp64 ? KCfg<double>::NT : KCfg<float>::NT),
-                                     args, smem, s);
+  const void* f = vec ? (const void*)k_krylov<float, true> : (const void*)k_krylov<float, false>;
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(KCfg<float>::NT), args, smem, s);
 }
 
 }  // namespace ed
