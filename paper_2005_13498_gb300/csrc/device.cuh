@@ -7,6 +7,23 @@
 
 namespace ed {
 
+// ---------------------------------------------------------------- host side
+// Lets `kernel` be launched with smem bytes of dynamic shared memory.  The
+// limit belongs to the function, for every context and thread of the process,
+// so it only ever takes one value, the most the device gives a block beside
+// the kernel's static arrays: set to what one sector needs, it would refuse
+// the launches another context was prepared for.
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, size_t smem) {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  const int64_t most = 227 * 1024 - (int64_t)fa.sharedSizeBytes;
+  if ((int64_t)smem > most) return cudaErrorInvalidValue;
+  if (fa.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // ---------------------------------------------------------------- utilities
 template <typename R> struct C2T;
 template <> struct C2T<float> { using T = float2; };

@@ -2023,27 +2023,18 @@ template <typename R, int NR, int PP, int MINB, bool SPLIT, int PPC, int MINBC, 
           int TMA, int NT, bool MV>
 static cudaError_t prepare_apply_t(const LaunchShape& sh) {
   constexpr bool V = sizeof(R) == 4;
-  const int sm = (int)sh.smem;
-  cudaError_t e = cudaFuncSetAttribute(k_apply<R, NR, PP, false, MINB, SPLIT, TMA, NT, MV>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  cudaError_t e = allow_smem(k_apply<R, NR, PP, false, MINB, SPLIT, TMA, NT, MV>, sh.smem);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_apply<R, NR, PP, V, MINB, SPLIT, TMA, NT, MV>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  e = allow_smem(k_apply<R, NR, PP, V, MINB, SPLIT, TMA, NT, MV>, sh.smem);
   if (e != cudaSuccess) return e;
   if constexpr (SPLIT && CB == 0) {
-    const int smc = (int)sh.smem_c;
-    e = cudaFuncSetAttribute(k_apply_tup<R, PPC, false, MINBC>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smc);
+    e = allow_smem(k_apply_tup<R, PPC, false, MINBC>, sh.smem_c);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_apply_tup<R, PPC, V, MINBC>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smc);
+    e = allow_smem(k_apply_tup<R, PPC, V, MINBC>, sh.smem_c);
   } else if constexpr (SPLIT) {
-    const int smc = (int)sh.smem_c;
-    e = cudaFuncSetAttribute(k_apply_up<R, PPC, false, MINBC, CB, TC>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smc);
+    e = allow_smem(k_apply_up<R, PPC, false, MINBC, CB, TC>, sh.smem_c);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_apply_up<R, PPC, V, MINBC, CB, TC>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, smc);
+    e = allow_smem(k_apply_up<R, PPC, V, MINBC, CB, TC>, sh.smem_c);
   }
   return e;
 }
@@ -2152,14 +2143,12 @@ static cudaError_t permute_cols(bool fp64, const void* src, void* dst, int dim_u
   if (smem > 227 * 1024) return cudaErrorInvalidValue;
   cudaError_t e;
   if (fp64) {
-    e = cudaFuncSetAttribute(k_permute_cols<double2>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(k_permute_cols<double2>, smem);
     if (e != cudaSuccess) return e;
     k_permute_cols<double2><<<dim_up, 256, smem, s>>>(static_cast<const double2*>(src),
                                                       static_cast<double2*>(dst), dim_dn, g);
   } else {
-    e = cudaFuncSetAttribute(k_permute_cols<float2>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_smem(k_permute_cols<float2>, smem);
     if (e != cudaSuccess) return e;
     k_permute_cols<float2><<<dim_up, 256, smem, s>>>(static_cast<const float2*>(src),
                                                      static_cast<float2*>(dst), dim_dn, g);

@@ -132,7 +132,8 @@ int apply_small_config(bool fp64, int64_t rows);
 // The default configuration (first candidate).
 LaunchShape apply_shape(int max_dim_up, int max_dim_dn, bool fp64, int n_groups);
 // Raise the dynamic shared-memory limit of the apply kernel for this shape
-// (once, before launches or graph capture).
+// (once, before launches or graph capture); cudaErrorInvalidValue when the
+// shape needs more than a block can have.
 cudaError_t prepare_apply(bool fp64, const LaunchShape& sh);
 
 // j >= 1: Lanczos step j; j == 0: plain apply x1 -> w with coefs row 0;

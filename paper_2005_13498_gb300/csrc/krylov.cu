@@ -830,12 +830,9 @@ size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups) {
 
 template <typename R, bool VEC>
 static cudaError_t prepare_t(size_t smem, int* ctas) {
-  cudaFuncAttributes fa;
-  cudaError_t e = cudaFuncGetAttributes(&fa, k_krylov<R, VEC>);
-  if (e != cudaSuccess) return e;
   *ctas = 0;
-  if (smem + fa.sharedSizeBytes > 227 * 1024) return cudaSuccess;
-  e = cudaFuncSetAttribute(k_krylov<R, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(k_krylov<R, VEC>, smem);
+  if (e == cudaErrorInvalidValue) return cudaSuccess;   // too large
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_krylov<R, VEC>, KCfg<R>::NT, smem);
 }
