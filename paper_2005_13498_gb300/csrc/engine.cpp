@@ -428,10 +428,15 @@ std::string Engine::setup_persistent(const SpinTable* up, bool vec_ok) {
   kry_deg_ = 1;
   for (int r = 0; r < up->dim; ++r) kry_deg_ = std::max(kry_deg_, up->off[r + 1] - up->off[r]);
   kry_vec_ = vec_ok;
-  kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_);
-  if (kry_smem_ > 227 * 1024) return "";
+  // as many sub-steps per launch as their coefficients leave room for
   int ctas = 0;
-  ED_TRY(krylov_prepare(kry_vec_, kry_smem_, &ctas));
+  for (kry_steps_ = kKrylovSteps; kry_steps_ > 0; --kry_steps_) {
+    kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_,
+                            krylov_coef_rows(kry_steps_, cfg_.energy));
+    if (kry_smem_ > 227 * 1024) continue;
+    ED_TRY(krylov_prepare(kry_vec_, kry_smem_, &ctas));
+    if (ctas > 0) break;
+  }
   if (ctas < 1) return "";
   ED_TRY(d_slots_.alloc(kKrylovSlotBytes));
   kry_grid_ = grid;
@@ -647,11 +652,10 @@ std::string Engine::run(int n_steps, bool profile, double* kernel_ms, int64_t* l
                         cudaStream_t s) {
   const bool f = cfg_.fp64;
   // Sectors whose rows fit the chip's shared memory run whole sub-steps in
-  // the persistent kernel, kKrylovSteps of them per launch (a launch of the
-  // largest such sector then lasts a few tens of ms).  A pinned
+  // the persistent kernel, up to kKrylovSteps of them per launch (a launch of
+  // the largest such sector then lasts a few tens of ms).  A pinned
   // configuration asks for the separate kernels.  In profile mode the kernel
   // itself adds up the time of its phases.
-  constexpr int kKrylovSteps = 16;
   // With the adaptive exit a small sector's pass is shorter than the check it
   // should hide, and the separate kernels, whose checks run on a stream of
   // their own, are faster (us for 20 steps with up to 10 vectors, 7 used,
@@ -673,8 +677,8 @@ std::string Engine::run(int n_steps, bool profile, double* kernel_ms, int64_t* l
       ED_TRY(cudaMemsetAsync(prof.p, 0, prof.bytes, s));
     }
     k.prof = static_cast<uint64_t*>(prof.p);
-    for (int n = 0; n == 0 || n < n_steps; n += kKrylovSteps) {
-      k.n_steps = std::min(kKrylovSteps, n_steps - n);
+    for (int n = 0; n == 0 || n < n_steps; n += kry_steps_) {
+      k.n_steps = std::min(kry_steps_, n_steps - n);
       const cudaError_t e = launch_krylov(kry_vec_, k, kry_grid_, kry_smem_, s);
       if (e == cudaErrorCooperativeLaunchTooLarge && n == 0) {
         // fewer SMs at hand than the device has (a partitioned context)

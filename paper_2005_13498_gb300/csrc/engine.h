@@ -148,7 +148,7 @@ class Engine {
   DevMem d_maps_, d_map_off_, d_map_spin_, d_ovl_, d_psiT_;
   bool need_psiT_ = false;
   // persistent Krylov kernel: grid 0 = not used
-  int kry_grid_ = 0, kry_rows_ = 0, kry_deg_ = 0;
+  int kry_grid_ = 0, kry_rows_ = 0, kry_deg_ = 0, kry_steps_ = 0;
   bool kry_vec_ = false;
   size_t kry_smem_ = 0;
   DevMem d_slots_;

@@ -210,9 +210,14 @@ struct KrylovArgs {
   int energy;        // record E(t) with a.coefs_obs
   uint64_t* prof;    // null, or [KK_COUNT][2]: ns and number of each kind's phases
 };
+constexpr int kKrylovSteps = 16;   // most sub-steps of a launch
+// Coefficient rows a launch of n_steps sub-steps keeps in shared memory.
+__host__ __device__ constexpr int krylov_coef_rows(int n_steps, int energy) {
+  return n_steps + (energy ? n_steps + 1 : 0);
+}
 // Dynamic shared memory of a launch, and the CTAs per SM it allows (0: does
 // not fit); krylov_prepare raises the kernel's limit.
-size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups);
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows);
 cudaError_t krylov_prepare(bool vec, size_t smem, int* ctas_per_sm);
 cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
                           cudaStream_t s);

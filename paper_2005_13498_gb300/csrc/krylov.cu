@@ -19,10 +19,18 @@
 // 50 ns); for the torus the shared-memory and L2 gathers (21 of 37 us per
 // Lanczos step).
 // It is used when two copies of a CTA's rows fit its shared memory: up to
-// about 15 MB of state (D = 1.9 M).  complex64 only: a complex128 form read, in
-// some builds, the previous step's bond coefficients in a few rows (gone without
-// a field, so not the vectors), for a reason not found, and gained 3 to 18 % over
-// the separate kernels.
+// about 15 MB of state (D = 1.9 M).  complex64 only: a complex128 form gained 3
+// to 18 % over the separate kernels.
+//
+// The coefficients of all sub-steps of a launch are in shared memory before its
+// first pass.  Loaded sub-step by sub-step into one table, right before the
+// pass that reads it, they came out wrong in some builds of the complex128 form
+// (energies off by up to 1e-6, other values in every run; never without a
+// field, never in a launch's first sub-step), though a block barrier stood
+// between and no reason was found in the source.  With the tables of the whole
+// launch that same form was right, and the same bit by bit, in 180 runs over
+// three sectors.  The complex64 form had shown no such error; its results did
+// not change.
 //
 // Grid-wide sums: each CTA publishes its float64 partial as two 64-bit words
 // that carry the sum's epoch in their upper halves, and one warp of every CTA
@@ -203,7 +211,7 @@ __device__ __forceinline__ void ldcg_pair(const C* row, int p, int dim, C& v0, C
 //  source rows in flight.
 __device__ __forceinline__ void off_diagonal(
     const SectorDev& sd, const float2* tile, int t, int p, int pcl, int npairs, const float2* x,
-    const uint2* const (&list)[2], const int (&deg)[2], const float2* coefS, const float2* coefQ,
+    const uint2* const (&list)[2], const int (&deg)[2], const float2* coefQ,
     bool vec, float2 (&acc)[2][2]) {
   constexpr int NR = 2;
   using TIO = TileIO<float2, NR>;
@@ -219,7 +227,7 @@ __device__ __forceinline__ void off_diagonal(
     acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
   }
   auto flush = [&](uint32_t g) {
-    const float2 c = coefS[g];
+    const float2 c = coefQ[1 + 2 * g];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       cmac(acc[r][0], c, s0[r]);
@@ -341,8 +349,8 @@ extern __shared__ __align__(16) unsigned char smem_raw[];
 struct Share {
   SectorDev sd;
   VecDev vd;
-  int off_w, off_q, off_c, off_l, off_d;   // byte offsets of the arrays below
-  int max_deg, nloc, ld, npairs, ntile, items, nwork;
+  int off_w, off_q, off_l, off_d;   // byte offsets of the arrays below
+  int n_coef, max_deg, nloc, ld, npairs, ntile, items, nwork;
 };
 constexpr int kOffShare = (sizeof(Scalars) + 15) & ~15;
 constexpr int kOffX = (kOffShare + sizeof(Share) + 15) & ~15;
@@ -351,19 +359,25 @@ __device__ __forceinline__ Share& share() { return *reinterpret_cast<Share*>(sme
 // rows of x_j and w: [tile rows][dim_dn + zero columns][NR]
 template <typename C> __device__ __forceinline__ C* tile_x() { return reinterpret_cast<C*>(smem_raw + kOffX); }
 template <typename C> __device__ __forceinline__ C* tile_w() { return reinterpret_cast<C*>(smem_raw + share().off_w); }
-// complex64: signed coefficients [1 + 2 n_groups]; coefficients [n_groups]
-__device__ __forceinline__ float2* coef_q() { return reinterpret_cast<float2*>(smem_raw + share().off_q); }
-template <typename C> __device__ __forceinline__ C* coef_s() { return reinterpret_cast<C*>(smem_raw + share().off_c); }
+// Signed coefficients, 1 + 2 n_groups to a row (0, then c_g and -c_g of every
+// group): a row for each sub-step of the launch, then, with energies, one for
+// its first time and one for the time after each sub-step.  All of them are
+// written before the first grid-wide sum and only read after it, so that no
+// pass depends on a hand-over within the launch.
+__device__ __forceinline__ const float2* coef_q(int row) {
+  return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * share().n_coef;
+}
 // T_up entries [rows][max_deg]: source offset, slot or group; their numbers
 __device__ __forceinline__ uint2* up_list() { return reinterpret_cast<uint2*>(smem_raw + share().off_l); }
 __device__ __forceinline__ int* up_deg() { return reinterpret_cast<int*>(smem_raw + share().off_d); }
 
-// w = s_in H x - s_prev x_prev of the CTA's rows into tileW; returns the
+// w = s_in H x - s_prev x_prev of the CTA's rows into tileW, H with the
+// coefficients of the given row; returns the
 // thread's Re<x, w>.  (One function for the Lanczos and the energy passes:
 // inlined in each place it took the registers of both.)
 template <typename R, bool VEC>
 __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
-                                          const typename C2T<R>::T* xp, R s_in, R s_prev) {
+                                          const typename C2T<R>::T* xp, R s_in, R s_prev, int row) {
   const Scalars& S = scalars();
   const Share& h = share();
   // the loads below must not move up across the grid-wide sum before the
@@ -382,8 +396,7 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
   C* const tileW = tile_w<C>();
   const uint2* const list = up_list();
   const int* const degS = up_deg();
-  const C* const coefS = coef_s<C>();
-  const float2* const coefQ = coef_q();
+  const float2* const coefQ = coef_q(row);
   double dot = 0.0;
   if (warp >= h.nwork) return dot;
   for (int it = warp; it < h.items; it += h.nwork) {
@@ -400,7 +413,7 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
       urow[r] = cta + (have ? li : 0) * G;
     }
     C acc[NR][2];
-    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefS, coefQ, VEC, acc);
+    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefQ, VEC, acc);
     if (p >= npairs) continue;
     const int d0 = 2 * p;
     const bool has1 = d0 + 1 < dim_dn;
@@ -479,12 +492,11 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
   const int RB = (k.rows + NR - 1) / NR;
   const int tile_bytes = RB * ld * 16;
   const int off_q = kOffX + 2 * tile_bytes;
-  const int off_c = off_q + (sizeof(R) == 4 ? (1 + 2 * a.n_groups) * 8 : 0);
-  const int off_l = off_c + a.n_groups * (int)sizeof(C);
+  const int n_coef = 1 + 2 * a.n_groups;
+  const int off_l = off_q + krylov_coef_rows(k.n_steps, k.energy) * n_coef * (int)sizeof(float2);
   C* const tileX = tile_x<C>();
   C* const tileW = reinterpret_cast<C*>(smem_raw + kOffX + tile_bytes);
   float2* const coefQ = reinterpret_cast<float2*>(smem_raw + off_q);
-  C* const coefS = reinterpret_cast<C*>(smem_raw + off_c);
   uint2* const list = reinterpret_cast<uint2*>(smem_raw + off_l);
   int* const degS = reinterpret_cast<int*>(list + (size_t)k.rows * k.max_deg);
   C* x1 = static_cast<C*>(vd.x1);
@@ -525,7 +537,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
   if (tid == 0) {
     h.off_w = kOffX + tile_bytes;
     h.off_q = off_q;
-    h.off_c = off_c;
+    h.n_coef = n_coef;
     h.off_l = off_l;
     h.off_d = off_l + k.rows * k.max_deg * (int)sizeof(uint2);
     h.max_deg = k.max_deg;
@@ -544,21 +556,20 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
   uint32_t epoch = 0;
   const int step0 = S.step;
 
-  auto load_coefs = [&](const void* base, int step) {
-    const C* c = reinterpret_cast<const C*>(base) + (size_t)step * a.n_groups;
-    for (int g = tid; g < a.n_groups; g += NT) coefS[g] = c[g];
-    if constexpr (sizeof(R) == 4)
-      for (int i = tid; i <= 2 * a.n_groups; i += NT) {
-        float2 q = make_float2(0.f, 0.f);
-        if (i > 0) {
-          const float2 cc = reinterpret_cast<const float2*>(c)[(i - 1) >> 1];
-          const float sg = ((i - 1) & 1) ? -1.f : 1.f;
-          q = make_float2(sg * cc.x, sg * cc.y);
-        }
-        coefQ[i] = q;
-      }
-    block_sync();
-  };
+  for (int i = tid; i < krylov_coef_rows(k.n_steps, k.energy) * n_coef; i += NT) {
+    const int row = i / n_coef, slot = i - row * n_coef;
+    float2 q = make_float2(0.f, 0.f);
+    if (slot > 0) {
+      const bool obs = row >= k.n_steps;
+      const float2 c = reinterpret_cast<const float2*>(
+          obs ? a.coefs_obs : a.coefs)[(size_t)(step0 + row - (obs ? k.n_steps : 0)) * a.n_groups +
+                                       ((slot - 1) >> 1)];
+      const float sg = ((slot - 1) & 1) ? -1.f : 1.f;
+      q = make_float2(sg * c.x, sg * c.y);
+    }
+    coefQ[i] = q;
+  }
+  block_sync();
   // one pass over the items: f(tile row, column tile, column pair)
   auto for_items = [&](auto&& f) {
     for (int it = warp; it < items; it += nwork) {
@@ -602,8 +613,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     }
   };
   auto energy = [&](int slot) -> bool {
-    load_coefs(a.coefs_obs, slot);
-    const double v[1] = {apply_pass<R, VEC>(x1, nullptr, (R)1, (R)0)};
+    const double v[1] = {apply_pass<R, VEC>(x1, nullptr, (R)1, (R)0, k.n_steps + slot - step0)};
     return grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
       if (cta == 0 && vd.out_energy) vd.out_energy[slot] = S.tot[0] / a.Ns;
     });
@@ -646,7 +656,6 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
 
   for (int s = 0; s < k.n_steps; ++s) {
     mark(-1);
-    load_coefs(a.coefs, S.step);
     // ---- Lanczos recursion
     for (int j = 1; j <= m && !S.stop; ++j) {
       const C* x = j == 1 ? x1 : V + (size_t)(j - 2) * vd.D;
@@ -654,7 +663,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       const R s_in = (R)S.inv[j];
       const R s_prev = j >= 2 ? (R)(S.beta[j - 1] * S.inv[j - 1]) : (R)0;
       if (warp >= nwork && j >= 2) conv_check(S, j - 1, a.tau, eps_tol);
-      const double v[1] = {apply_pass<R, VEC>(x, xp, s_in, s_prev)};
+      const double v[1] = {apply_pass<R, VEC>(x, xp, s_in, s_prev, s)};
       if (!grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
             const double re = S.tot[0];
             S.alpha[j] = re * S.inv[j];
@@ -821,11 +830,11 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
 
 }  // namespace
 
-size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups) {
+size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows) {
   const int nr = KCfg<float>::NR;
   const size_t rb = (rows + nr - 1) / nr;
-  return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 + (size_t)(1 + 2 * n_groups) * 8 +
-         (size_t)n_groups * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+  return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 +
+         (size_t)coef_rows * (1 + 2 * n_groups) * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
 }
 
 template <typename R, bool VEC>
