@@ -329,8 +329,6 @@ __device__ __forceinline__ bool same(double a, double b) {
 // in the caller's coefficients.  With the T_up additions and the
 // products selected by short conditional blocks the compiler predicated them,
 // and switched-off instructions take the pipe's time as well: 1.94 ms.
-// lo, hi: which of the lane's two columns to compute
-// (uniform over the warp).
 __device__ __forceinline__ void ldcg2(const double2* row, int p, int dim, double2& v0, double2& v1) {
   v0 = __ldcg(row + 2 * p);
   v1 = czero<double2>();
@@ -340,8 +338,7 @@ __device__ __forceinline__ void ldcg2(const double2* row, int p, int dim, double
 template <typename Get>
 __device__ __forceinline__ void off_diagonal_c128(const SectorDev& sd, const double2* tile, int t,
                                                   int pcl, const double2* x, int ne, Get&& get,
-                                                  const double2* coefS, bool lo, bool hi,
-                                                  double2 (&acc)[2]) {
+                                                  const double2* coefS, double2 (&acc)[2]) {
   using C = double2;
   using TIO = TileIO<C, 1>;
   const int lane = threadIdx.x & 31;
@@ -356,11 +353,11 @@ __device__ __forceinline__ void off_diagonal_c128(const SectorDev& sd, const dou
   C s0 = czero<C>(), s1 = s0, cur = s0;
   acc[0] = acc[1] = s0;
   auto flush = [&]() {
-    if (lo) { acc[0].x += cur.x * s0.x; acc[0].y += cur.x * s0.y; }
-    if (hi) { acc[1].x += cur.x * s1.x; acc[1].y += cur.x * s1.y; }
+    acc[0].x += cur.x * s0.x; acc[0].y += cur.x * s0.y;
+    acc[1].x += cur.x * s1.x; acc[1].y += cur.x * s1.y;
     if (!is_zero(cur.y)) {   // uniform over the block
-      if (lo) { acc[0].x -= cur.y * s0.y; acc[0].y += cur.y * s0.x; }
-      if (hi) { acc[1].x -= cur.y * s1.y; acc[1].y += cur.y * s1.x; }
+      acc[0].x -= cur.y * s0.y; acc[0].y += cur.y * s0.x;
+      acc[1].x -= cur.y * s1.y; acc[1].y += cur.y * s1.x;
     }
   };
   bool any = false;
@@ -403,14 +400,14 @@ __device__ __forceinline__ void off_diagonal_c128(const SectorDev& sd, const dou
       C a0[1], a1[1];
       TIO::load_off(tile, o0, a0);
       TIO::load_off(tile, o1, a1);
-      if (lo) cax(s0, g0, a0[0]);
-      if (hi) cax(s1, g1, a1[0]);
+      cax(s0, g0, a0[0]);
+      cax(s1, g1, a1[0]);
     }
     // one branch per count: short conditional blocks become predicated
     // instructions, and those take the pipe's time also when switched off
     auto add = [&](int i) {
-      if (lo) cax(s0, sg[i], v[i][0]);
-      if (hi) cax(s1, sg[i], v[i][1]);
+      cax(s0, sg[i], v[i][0]);
+      cax(s1, sg[i], v[i][1]);
     };
     switch (nb) {
       case 1: add(0); break;
@@ -425,8 +422,8 @@ __device__ __forceinline__ void off_diagonal_c128(const SectorDev& sd, const dou
       C u0, u1;
       ldcg2(x + m.x, pcl, dim_dn, u0, u1);
       const double s = (m.y >> 31) ? -1.0 : 1.0;
-      if (lo) cax(s0, s, u0);
-      if (hi) cax(s1, s, u1);
+      cax(s0, s, u0);
+      cax(s1, s, u1);
       ++e;
     }
     ge = e < ne ? get(e).y & 0xFFu : kEnd;

@@ -623,7 +623,7 @@ k_apply(BatchArgs a, int j) {
                             return make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
                                               ((en >> kEntGroupShift) & 0xFFu) | (en & kEntSignBit));
                           },
-                          coefS, true, true, acc[0]);
+                          coefS, acc[0]);
     }
 #pragma unroll
     for (int k = 0; k < (LEAN ? 0 : PP); ++k) {

@@ -51,9 +51,10 @@ constexpr int kErrNumeric = 7;    // ED_ERR_NUMERIC
 constexpr int kUpBatch = 6;
 constexpr int kPollLanes = (kKrylovMaxGrid + 31) / 32;
 
-// two rows per 16-byte tile column, 20 warps at 96 registers
-template <typename R> struct KCfg;
-template <> struct KCfg<float> { static constexpr int NT = 640, NR = 2; };
+// two rows per 16-byte tile column, 20 warps at 96 registers (980 bytes of
+// spill stores and 1628 of spill loads in the code of the paired form)
+constexpr int NT = 640, NR = 2;
+using TIO = TileIO<float2, NR>;
 
 // Scalars of the Lanczos recursion in shared memory, 1-based as LanczosState.
 struct Scalars {
@@ -90,7 +91,7 @@ __device__ __forceinline__ void st_slot(ulonglong2* p, double v, uint32_t epoch)
 // CTA; `after` runs in thread 0 with the totals in place, before the other
 // threads go on.  DATA: vectors written before the call are read by other
 // CTAs after it.  False when a wait gave up (in all threads of the CTA).
-template <int K, bool DATA, int NT, typename F>
+template <int K, bool DATA, typename F>
 __device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Scalars& S,
                                          const KrylovArgs& k, uint32_t& epoch, F&& after) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -172,9 +173,10 @@ __device__ __forceinline__ bool grid_sum(const double (&v)[K], double* redS, Sca
 }
 
 // L2 loads of the column pair (2p, 2p+1) of a row: the vectors are written by
-// other SMs during the kernel, so nothing may come from L1.  SELF: the pair
-// may have been written by this thread since the last call of a function that
-// is not inlined; such loads are volatile and stay behind those stores.
+// other SMs during the kernel, so nothing may come from L1.  SELF: the pair is
+// one this thread wrote earlier in the kernel.  __ldcg tells the compiler
+// nothing about the memory it reads, so it may be moved ahead of a store to the
+// same address; these loads name the memory and stay behind it.
 template <typename T4>
 __device__ __forceinline__ T4 ldl2(const T4* p) {
   static_assert(sizeof(T4) == 16 || sizeof(T4) == 8, "16- or 8-byte loads");
@@ -191,30 +193,29 @@ __device__ __forceinline__ T4 ldl2(const T4* p) {
   }
   return v;
 }
-template <typename C, bool VEC, bool SELF>
-__device__ __forceinline__ void ldcg_pair(const C* row, int p, int dim, C& v0, C& v1) {
+template <bool VEC, bool SELF>
+__device__ __forceinline__ void ldcg_pair(const float2* row, int p, int dim, float2& v0, float2& v1) {
   if constexpr (VEC) {
     const float4* a = reinterpret_cast<const float4*>(row) + p;
     const float4 f = SELF ? ldl2(a) : __ldcg(a);
     v0.x = f.x; v0.y = f.y; v1.x = f.z; v1.y = f.w;
   } else {
     v0 = SELF ? ldl2(row + 2 * p) : __ldcg(row + 2 * p);
-    v1 = czero<C>();
+    v1 = make_float2(0.f, 0.f);
     if (2 * p + 1 < dim) v1 = SELF ? ldl2(row + 2 * p + 1) : __ldcg(row + 2 * p + 1);
   }
 }
 
 // The off-diagonal part of H x for one item, NR tile rows x 64 columns (two
-// columns per lane): acc[r][h] of row r and column 2 p + h.
-// T_dn over the ELL slots of the tile (two slots per turn, words
-//  a turn ahead), then T_up row by row with the signed coefficients, kUpBatch
-//  source rows in flight.
+// columns per lane): acc[r][h] of row r and column 2 p + h (pcl: the pair p,
+// clamped to the row).  T_dn over the ELL slots of the tile (two slots per turn,
+// words a turn ahead), then T_up row by row with the signed coefficients,
+// kUpBatch source rows in flight.
+template <bool VEC>
 __device__ __forceinline__ void off_diagonal(
-    const SectorDev& sd, const float2* tile, int t, int p, int pcl, int npairs, const float2* x,
-    const uint2* const (&list)[2], const int (&deg)[2], const float2* coefQ,
-    bool vec, float2 (&acc)[2][2]) {
-  constexpr int NR = 2;
-  using TIO = TileIO<float2, NR>;
+    const SectorDev& sd, const float2* tile, int t, int pcl, const float2* x,
+    const uint2* const (&list)[NR], const int (&deg)[NR], const float2* coefQ,
+    float2 (&acc)[NR][2]) {
   const int lane = threadIdx.x & 31;
   const int dim_dn = sd.dim_dn;
   const int q0 = __ldg(sd.dn_tslot_off + t), q1 = __ldg(sd.dn_tslot_off + t + 1);
@@ -278,9 +279,7 @@ __device__ __forceinline__ void off_diagonal(
         if (e + i < deg[r]) {   // uniform over the warp
           const uint2 en = list[r][e + i];
           cs[i] = en.y;
-          const float2* src = x + en.x;
-          if (vec) ldcg_pair<float2, true, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
-          else ldcg_pair<float2, false, false>(src, pcl, dim_dn, v[i][0], v[i][1]);
+          ldcg_pair<VEC, false>(x + en.x, pcl, dim_dn, v[i][0], v[i][1]);
         }
 #pragma unroll
       for (int i = 0; i < NB; ++i)
@@ -357,8 +356,8 @@ constexpr int kOffX = (kOffShare + sizeof(Share) + 15) & ~15;
 __device__ __forceinline__ Scalars& scalars() { return *reinterpret_cast<Scalars*>(smem_raw); }
 __device__ __forceinline__ Share& share() { return *reinterpret_cast<Share*>(smem_raw + kOffShare); }
 // rows of x_j and w: [tile rows][dim_dn + zero columns][NR]
-template <typename C> __device__ __forceinline__ C* tile_x() { return reinterpret_cast<C*>(smem_raw + kOffX); }
-template <typename C> __device__ __forceinline__ C* tile_w() { return reinterpret_cast<C*>(smem_raw + share().off_w); }
+__device__ __forceinline__ float2* tile_x() { return reinterpret_cast<float2*>(smem_raw + kOffX); }
+__device__ __forceinline__ float2* tile_w() { return reinterpret_cast<float2*>(smem_raw + share().off_w); }
 // Signed coefficients, 1 + 2 n_groups to a row (0, then c_g and -c_g of every
 // group): a row for each sub-step of the launch, then, with energies, one for
 // its first time and one for the time after each sub-step.  All of them are
@@ -367,33 +366,29 @@ template <typename C> __device__ __forceinline__ C* tile_w() { return reinterpre
 __device__ __forceinline__ const float2* coef_q(int row) {
   return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * share().n_coef;
 }
-// T_up entries [rows][max_deg]: source offset, slot or group; their numbers
+// T_up entries [rows][max_deg]: source offset, coefficient slot; their numbers
 __device__ __forceinline__ uint2* up_list() { return reinterpret_cast<uint2*>(smem_raw + share().off_l); }
 __device__ __forceinline__ int* up_deg() { return reinterpret_cast<int*>(smem_raw + share().off_d); }
 
 // w = s_in H x - s_prev x_prev of the CTA's rows into tileW, H with the
-// coefficients of the given row; returns the
-// thread's Re<x, w>.  (One function for the Lanczos and the energy passes:
-// inlined in each place it took the registers of both.)
-template <typename R, bool VEC>
-__device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
-                                          const typename C2T<R>::T* xp, R s_in, R s_prev, int row) {
+// coefficients of the given row; returns the thread's Re<x, w>.  Inlined in the
+// Lanczos loop and in the energies.
+template <bool VEC>
+__device__ __forceinline__ double apply_pass(const float2* x, const float2* xp, float s_in,
+                                             float s_prev, int row) {
   const Scalars& S = scalars();
   const Share& h = share();
   // the loads below must not move up across the grid-wide sum before the
   // pass: they depend on pointers that are opaque from here on
   asm volatile("" : "+l"(x) : : "memory");
   asm volatile("" : "+l"(xp) : : "memory");
-  using C = typename C2T<R>::T;
-  constexpr int NR = KCfg<R>::NR;
-  using TIO = TileIO<C, NR>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int G = gridDim.x, cta = blockIdx.x;
   const SectorDev& sd = h.sd;
   const int dim_dn = sd.dim_dn, npairs = h.npairs, ntile = h.ntile, nloc = h.nloc;
   const int pitch = h.ld * NR;
-  const C* const tileX = tile_x<C>();
-  C* const tileW = tile_w<C>();
+  const float2* const tileX = tile_x();
+  float2* const tileW = tile_w();
   const uint2* const list = up_list();
   const int* const degS = up_deg();
   const float2* const coefQ = coef_q(row);
@@ -401,7 +396,7 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
   if (warp >= h.nwork) return dot;
   for (int it = warp; it < h.items; it += h.nwork) {
     const int b = it / ntile, t = it - b * ntile, p = 32 * t + lane;
-    const C* tile = tileX + b * pitch;
+    const float2* tile = tileX + b * pitch;
     const uint2* lst[NR];
     int deg[NR], urow[NR];
 #pragma unroll
@@ -412,36 +407,36 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
       deg[r] = have ? degS[li] : 0;
       urow[r] = cta + (have ? li : 0) * G;
     }
-    C acc[NR][2];
-    off_diagonal(sd, tile, t, p, min(p, npairs - 1), npairs, x, lst, deg, coefQ, VEC, acc);
+    float2 acc[NR][2];
+    off_diagonal<VEC>(sd, tile, t, min(p, npairs - 1), x, lst, deg, coefQ, acc);
     if (p >= npairs) continue;
     const int d0 = 2 * p;
     const bool has1 = d0 + 1 < dim_dn;
     const uint32_t dw0 = __ldg(sd.dn_word + d0), dw1 = has1 ? __ldg(sd.dn_word + d0 + 1) : 0u;
-    C xa[NR], xb[NR], oa[NR], ob[NR];
+    float2 xa[NR], xb[NR], oa[NR], ob[NR];
     TIO::load(tile, d0, xa);
     TIO::load(tile, d0 + 1, xb);
-    R da = (R)0;
+    float da = 0.f;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      oa[r] = ob[r] = czero<C>();
+      oa[r] = ob[r] = make_float2(0.f, 0.f);
       if (b * NR + r >= nloc) continue;
       const uint32_t uw = __ldg(sd.up_word + urow[r]);
-      R g0 = (R)S.utab[__popc(uw & dw0)], g1 = (R)S.utab[__popc(uw & dw1)];
+      float g0 = (float)S.utab[__popc(uw & dw0)], g1 = (float)S.utab[__popc(uw & dw1)];
       if (sd.up_eps) {
-        const R eu = (R)__ldg(sd.up_eps + urow[r]);
-        g0 += eu + (R)__ldg(sd.dn_eps + d0);
-        g1 += eu + (has1 ? (R)__ldg(sd.dn_eps + d0 + 1) : (R)0);
+        const float eu = (float)__ldg(sd.up_eps + urow[r]);
+        g0 += eu + (float)__ldg(sd.dn_eps + d0);
+        g1 += eu + (has1 ? (float)__ldg(sd.dn_eps + d0 + 1) : 0.f);
       }
-      C a0 = acc[r][0], a1 = acc[r][1];
+      float2 a0 = acc[r][0], a1 = acc[r][1];
       a0.x += g0 * xa[r].x;
       a0.y += g0 * xa[r].y;
       a1.x += g1 * xb[r].x;
       a1.y += g1 * xb[r].y;
-      C o0, o1;
+      float2 o0, o1;
       if (xp) {
-        C p0, p1;
-        ldcg_pair<C, VEC, false>(xp + (size_t)urow[r] * dim_dn, p, dim_dn, p0, p1);
+        float2 p0, p1;
+        ldcg_pair<VEC, false>(xp + (size_t)urow[r] * dim_dn, p, dim_dn, p0, p1);
         o0.x = s_in * a0.x - s_prev * p0.x;
         o0.y = s_in * a0.y - s_prev * p0.y;
         o1.x = s_in * a1.x - s_prev * p1.x;
@@ -462,16 +457,14 @@ __device__ __forceinline__ double apply_pass(const typename C2T<R>::T* x,
   return dot;
 }
 
-template <typename R, bool VEC>
-__global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
-  using C = typename C2T<R>::T;
-  constexpr int NT = KCfg<R>::NT, NR = KCfg<R>::NR, NW = NT / 32;
-  using TIO = TileIO<C, NR>;
+template <bool VEC>
+__global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
+  constexpr int NW = NT / 32;
   Scalars& S = scalars();
   Share& h = share();
   __shared__ double redS[NT];
-  __shared__ C cf[kMaxKrylov + 1];
-  __shared__ C cf_lo;
+  __shared__ float2 cf[kMaxKrylov + 1];
+  __shared__ float2 cf_lo;
 
   const BatchArgs& a = k.a;
   if (threadIdx.x == 0) {
@@ -494,13 +487,13 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
   const int off_q = kOffX + 2 * tile_bytes;
   const int n_coef = 1 + 2 * a.n_groups;
   const int off_l = off_q + krylov_coef_rows(k.n_steps, k.energy) * n_coef * (int)sizeof(float2);
-  C* const tileX = tile_x<C>();
-  C* const tileW = reinterpret_cast<C*>(smem_raw + kOffX + tile_bytes);
+  float2* const tileX = tile_x();
+  float2* const tileW = reinterpret_cast<float2*>(smem_raw + kOffX + tile_bytes);
   float2* const coefQ = reinterpret_cast<float2*>(smem_raw + off_q);
   uint2* const list = reinterpret_cast<uint2*>(smem_raw + off_l);
   int* const degS = reinterpret_cast<int*>(list + (size_t)k.rows * k.max_deg);
-  C* x1 = static_cast<C*>(vd.x1);
-  C* V = static_cast<C*>(vd.V);
+  float2* x1 = static_cast<float2*>(vd.x1);
+  float2* V = static_cast<float2*>(vd.V);
   const int m = st->m;
   const double eps_tol = st->eps_tol;
   const int items = nblk * ntile;
@@ -515,23 +508,22 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       const uint32_t en = __ldg(sd.up_ent + e0 + i);
       const uint32_t g = (en >> kEntGroupShift) & 0xFFu;
       list[(size_t)li * k.max_deg + i] =
-          make_uint2((en & kEntRankMask) * (uint32_t)dim_dn,
-                     sizeof(R) == 4 ? 1u + 2u * g + (en >> 31) : g | (en & kEntSignBit));
+          make_uint2((en & kEntRankMask) * (uint32_t)dim_dn, 1u + 2u * g + (en >> 31));
     }
     if (tid == 0) degS[li] = ne;
   }
   for (int i = tid; i < RB * ld; i += NT) {
     const int b = i / ld, d = i - b * ld;
-    C v[NR];
+    float2 v[NR];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       const int li = b * NR + r;
-      v[r] = li < nloc && d < dim_dn ? ldl2(x1 + (size_t)(cta + li * G) * dim_dn + d) : czero<C>();
+      v[r] = li < nloc && d < dim_dn ? ldl2(x1 + (size_t)(cta + li * G) * dim_dn + d) : make_float2(0.f, 0.f);
     }
     TIO::store(tileX + (size_t)b * ld * NR, d, v);
-    C z[NR];
+    float2 z[NR];
 #pragma unroll
-    for (int r = 0; r < NR; ++r) z[r] = czero<C>();
+    for (int r = 0; r < NR; ++r) z[r] = make_float2(0.f, 0.f);
     TIO::store(tileW + (size_t)b * ld * NR, d, z);
   }
   if (tid == 0) {
@@ -579,19 +571,19 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     }
   };
   // psi -> per-thread |psi|^2 and sum of double occupancies of tile values
-  auto weigh = [&](int b, int p, const C (&va)[NR], const C (&vb)[NR], double& n2, double& dd) {
+  auto weigh = [&](int b, int p, const float2 (&va)[NR], const float2 (&vb)[NR], double& n2, double& dd) {
     const int d0 = 2 * p;
     const bool has1 = d0 + 1 < dim_dn;
     const uint32_t dw0 = __ldg(sd.dn_word + d0), dw1 = has1 ? __ldg(sd.dn_word + d0 + 1) : 0u;
-    R nl = (R)0, wl = (R)0;
+    float nl = 0.f, wl = 0.f;
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       if (b * NR + r >= nloc) continue;
       const uint32_t uw = __ldg(sd.up_word + cta + (b * NR + r) * G);
-      const R qa = va[r].x * va[r].x + va[r].y * va[r].y;
-      const R qb = has1 ? vb[r].x * vb[r].x + vb[r].y * vb[r].y : (R)0;
+      const float qa = va[r].x * va[r].x + va[r].y * va[r].y;
+      const float qb = has1 ? vb[r].x * vb[r].x + vb[r].y * vb[r].y : 0.f;
       nl += qa + qb;
-      wl += (R)__popc(uw & dw0) * qa + (R)__popc(uw & dw1) * qb;
+      wl += (float)__popc(uw & dw0) * qa + (float)__popc(uw & dw1) * qb;
     }
     n2 += (double)nl;
     dd += (double)wl;
@@ -613,8 +605,8 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     }
   };
   auto energy = [&](int slot) -> bool {
-    const double v[1] = {apply_pass<R, VEC>(x1, nullptr, (R)1, (R)0, k.n_steps + slot - step0)};
-    return grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
+    const double v[1] = {apply_pass<VEC>(x1, nullptr, 1.f, 0.f, k.n_steps + slot - step0)};
+    return grid_sum<1, false>(v, redS, S, k, epoch, [&]() {
       if (cta == 0 && vd.out_energy) vd.out_energy[slot] = S.tot[0] / a.Ns;
     });
   };
@@ -645,12 +637,12 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     double v[2] = {0.0, 0.0};
     for_items([&](int b, int t, int p) {
       if (p >= npairs) return;
-      C xa[NR], xb[NR];
+      float2 xa[NR], xb[NR];
       TIO::load(tileX + (size_t)b * ld * NR, 2 * p, xa);
       TIO::load(tileX + (size_t)b * ld * NR, 2 * p + 1, xb);
       weigh(b, p, xa, xb, v[0], v[1]);
     });
-    if (!grid_sum<2, true, NT>(v, redS, S, k, epoch, [&]() { new_state(step0); })) { finish(); return; }
+    if (!grid_sum<2, true>(v, redS, S, k, epoch, [&]() { new_state(step0); })) { finish(); return; }
     if (k.energy && step0 == 0 && !energy(0)) { finish(); return; }
   }
 
@@ -658,13 +650,13 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
     mark(-1);
     // ---- Lanczos recursion
     for (int j = 1; j <= m && !S.stop; ++j) {
-      const C* x = j == 1 ? x1 : V + (size_t)(j - 2) * vd.D;
-      const C* xp = j < 2 ? nullptr : j == 2 ? x1 : V + (size_t)(j - 3) * vd.D;
-      const R s_in = (R)S.inv[j];
-      const R s_prev = j >= 2 ? (R)(S.beta[j - 1] * S.inv[j - 1]) : (R)0;
+      const float2* x = j == 1 ? x1 : V + (size_t)(j - 2) * vd.D;
+      const float2* xp = j < 2 ? nullptr : j == 2 ? x1 : V + (size_t)(j - 3) * vd.D;
+      const float s_in = (float)S.inv[j];
+      const float s_prev = j >= 2 ? (float)(S.beta[j - 1] * S.inv[j - 1]) : 0.f;
       if (warp >= nwork && j >= 2) conv_check(S, j - 1, a.tau, eps_tol);
-      const double v[1] = {apply_pass<R, VEC>(x, xp, s_in, s_prev, s)};
-      if (!grid_sum<1, false, NT>(v, redS, S, k, epoch, [&]() {
+      const double v[1] = {apply_pass<VEC>(x, xp, s_in, s_prev, s)};
+      if (!grid_sum<1, false>(v, redS, S, k, epoch, [&]() {
             const double re = S.tot[0];
             S.alpha[j] = re * S.inv[j];
             S.as = S.alpha[j] * S.inv[j];
@@ -680,31 +672,31 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       mark(KK_APPLY);
       if (S.stop || j == m) break;
       // x_{j+1} = w - alpha_j s_j x_j, into the tile and V
-      const R as = (R)S.as;
-      C* xn = V + (size_t)(j - 1) * vd.D;
+      const float as = (float)S.as;
+      float2* xn = V + (size_t)(j - 1) * vd.D;
       double nrm[1] = {0.0};
       for_items([&](int b, int t, int p) {
         if (p >= npairs) return;
         const int d0 = 2 * p;
         const bool has1 = d0 + 1 < dim_dn;
-        C* tx = tileX + (size_t)b * ld * NR;
-        C xa[NR], xb[NR], wa[NR], wb[NR];
+        float2* tx = tileX + (size_t)b * ld * NR;
+        float2 xa[NR], xb[NR], wa[NR], wb[NR];
         TIO::load(tx, d0, xa);
         TIO::load(tx, d0 + 1, xb);
         TIO::load(tileW + (size_t)b * ld * NR, d0, wa);
         TIO::load(tileW + (size_t)b * ld * NR, d0 + 1, wb);
-        R nl = (R)0;
+        float nl = 0.f;
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-          C o0, o1;
+          float2 o0, o1;
           o0.x = wa[r].x - as * xa[r].x;
           o0.y = wa[r].y - as * xa[r].y;
-          o1.x = has1 ? wb[r].x - as * xb[r].x : (R)0;
-          o1.y = has1 ? wb[r].y - as * xb[r].y : (R)0;
+          o1.x = has1 ? wb[r].x - as * xb[r].x : 0.f;
+          o1.y = has1 ? wb[r].y - as * xb[r].y : 0.f;
           xa[r] = o0;
           xb[r] = o1;
           if (b * NR + r < nloc) {
-            store_pair<C, VEC>(xn + (size_t)(cta + (b * NR + r) * G) * dim_dn, p, dim_dn, o0, o1);
+            store_pair<float2, VEC>(xn + (size_t)(cta + (b * NR + r) * G) * dim_dn, p, dim_dn, o0, o1);
             nl += o0.x * o0.x + o0.y * o0.y + o1.x * o1.x + o1.y * o1.y;
           }
         }
@@ -712,7 +704,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
         if (has1) TIO::store(tx, d0 + 1, xb);
         nrm[0] += (double)nl;
       });
-      if (!grid_sum<1, true, NT>(nrm, redS, S, k, epoch, [&]() {
+      if (!grid_sum<1, true>(nrm, redS, S, k, epoch, [&]() {
             const double beta = sqrt(S.tot[0]);
             const double sc = fmax(S.scale, fabs(S.alpha[j]));
             S.beta[j] = beta;
@@ -766,11 +758,11 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       for (int i = lane; i < n; i += 32) {
         const double f = zero ? 0.0 : S.beta0 * S.inv[i + 1];
         const double re = f * S.yre[i], im = f * S.yim[i];
-        cf[i].x = (R)re;
-        cf[i].y = (R)im;
+        cf[i].x = (float)re;
+        cf[i].y = (float)im;
         if (i == 0) {
-          cf_lo.x = (R)(re - (double)(R)re);
-          cf_lo.y = (R)(im - (double)(R)im);
+          cf_lo.x = (float)(re - (double)(float)re);
+          cf_lo.y = (float)(im - (double)(float)im);
         }
       }
     block_sync();
@@ -786,28 +778,28 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       if (p >= npairs) return;
       const int d0 = 2 * p;
       const bool has1 = d0 + 1 < dim_dn;
-      C pa[NR], pb[NR];
+      float2 pa[NR], pb[NR];
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
-        pa[r] = pb[r] = czero<C>();
+        pa[r] = pb[r] = make_float2(0.f, 0.f);
         if (b * NR + r >= nloc) continue;
         const size_t off = (size_t)(cta + (b * NR + r) * G) * dim_dn;
-        C x0, x1v;
-        ldcg_pair<C, VEC, true>(x1 + off, p, dim_dn, x0, x1v);
-        C o0 = czero<C>(), o1 = czero<C>();
+        float2 x0, x1v;
+        ldcg_pair<VEC, true>(x1 + off, p, dim_dn, x0, x1v);
+        float2 o0 = make_float2(0.f, 0.f), o1 = make_float2(0.f, 0.f);
         cmac(o0, cf_lo, x0);
         cmac(o1, cf_lo, x1v);
-        const C* Vr = V + off;
+        const float2* Vr = V + off;
 #pragma unroll 8
         for (int jj = 1; jj < nv; ++jj) {
-          C y0, y1;
-          ldcg_pair<C, VEC, true>(Vr + (size_t)(jj - 1) * vd.D, p, dim_dn, y0, y1);
+          float2 y0, y1;
+          ldcg_pair<VEC, true>(Vr + (size_t)(jj - 1) * vd.D, p, dim_dn, y0, y1);
           cmac(o0, cf[jj], y0);
           cmac(o1, cf[jj], y1);
         }
         cmac(o0, cf[0], x0);
         cmac(o1, cf[0], x1v);
-        store_pair<C, VEC>(x1 + off, p, dim_dn, o0, o1);
+        store_pair<float2, VEC>(x1 + off, p, dim_dn, o0, o1);
         pa[r] = o0;
         pb[r] = o1;
       }
@@ -815,7 +807,7 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
       if (has1) TIO::store(tileX + (size_t)b * ld * NR, d0 + 1, pb);
       weigh(b, p, pa, pb, v[0], v[1]);
     });
-    if (!grid_sum<2, true, NT>(v, redS, S, k, epoch, [&]() {
+    if (!grid_sum<2, true>(v, redS, S, k, epoch, [&]() {
           S.step = S.step + 1;
           new_state(S.step);
         })) { finish(); return; }
@@ -831,23 +823,22 @@ __global__ void __launch_bounds__(KCfg<R>::NT, 1) k_krylov(KrylovArgs k) {
 }  // namespace
 
 size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows) {
-  const int nr = KCfg<float>::NR;
-  const size_t rb = (rows + nr - 1) / nr;
+  const size_t rb = (rows + NR - 1) / NR;
   return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 +
          (size_t)coef_rows * (1 + 2 * n_groups) * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
 }
 
-template <typename R, bool VEC>
+template <bool VEC>
 static cudaError_t prepare_t(size_t smem, int* ctas) {
   *ctas = 0;
-  const cudaError_t e = allow_smem(k_krylov<R, VEC>, smem);
+  const cudaError_t e = allow_smem(k_krylov<VEC>, smem);
   if (e == cudaErrorInvalidValue) return cudaSuccess;   // too large
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_krylov<R, VEC>, KCfg<R>::NT, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_krylov<VEC>, NT, smem);
 }
 
 cudaError_t krylov_prepare(bool vec, size_t smem, int* ctas_per_sm) {
-  return vec ? prepare_t<float, true>(smem, ctas_per_sm) : prepare_t<float, false>(smem, ctas_per_sm);
+  return vec ? prepare_t<true>(smem, ctas_per_sm) : prepare_t<false>(smem, ctas_per_sm);
 }
 
 cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
@@ -855,8 +846,8 @@ cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
   cudaError_t e = cudaMemsetAsync(k.slots, 0, kKrylovSlotBytes, s);
   if (e != cudaSuccess) return e;
   void* args[] = {const_cast<KrylovArgs*>(&k)};
-  const void* f = vec ? (const void*)k_krylov<float, true> : (const void*)k_krylov<float, false>;
-  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(KCfg<float>::NT), args, smem, s);
+  const void* f = vec ? (const void*)k_krylov<true> : (const void*)k_krylov<false>;
+  return cudaLaunchCooperativeKernel(f, dim3(grid), dim3(NT), args, smem, s);
 }
 
 }  // namespace ed
