@@ -172,7 +172,7 @@ std::string tune_apply(const ApplyTuneTarget& t, cudaStream_t s, LaunchShape* sh
     for (int d : t.dim_up) rows += d;
     *shape = cands.front();
     for (const LaunchShape& c : cands)
-      if (c.cfg == apply_small_config(t.fp64, rows)) *shape = c;
+      if (c.cfg == apply_small_config(t.fp64, rows, t.max_dim_dn)) *shape = c;
     build(*shape);
     std::lock_guard<std::mutex> lock(mu);
     cache[key] = shape->cfg;

@@ -1971,20 +1971,33 @@ std::vector<LaunchShape> apply_candidates(int max_dim_up, int max_dim_dn, bool f
   return out;
 }
 
-// One row per CTA while the rows fit two CTAs on each of the 152 SMs, then
-// the entries that hold more CTAs per SM: complex64 two rows per CTA, three
-// CTAs (912 rows in a wave) or four.  us per product of one vector, and of
-// three where marked, entries 0 / 1 / 2 / 3 in complex64 and 4 / 5 / 6 / 24 in
-// complex128:
-//    70 x 70    8.3 /  6.8 /  8.2 /  6.2    16.5 / 12.4 / 10.3 / 11.3
-//   210 x 210   9.3 /  8.2 /  8.2 /  6.2    18.5 / 13.4 / 12.3 / 12.4
-//   364 x 91   10.3 /  8.2 /  8.2 /  8.3    24.6 / 11.1 / 14.4 / 10.3
-//   462 x 330  10.3 /  8.3 /  8.3 / 10.3    36.0 / 24.7 / 26.7 / 24.6
-//   792 x 66   20.5 / 20.6 / 18.5 / 28.7     152 / 55.4 / 79.9 / 59.5  (three)
-//   924 x 924  20.5 / 22.6 / 20.6 / 26.7     211 /  156 /  151 /  153
-int apply_small_config(bool fp64, int64_t rows) {
+// One row per CTA while the rows fit two CTAs on each of the 152 SMs.  Then, in
+// complex64, two rows per CTA: three CTAs per SM with two column pairs per
+// thread (entry 1, 912 rows in a wave) or four with one pair (entry 2, 1216
+// rows, 512 columns at a time).  Rows longer than that take entry 2 through
+// its entry list once more; between 912 and 1216 of them fit one wave of four
+// rows per CTA, two CTAs per SM (entry 0), above that entry 1 is ahead again.
+// us per product of one vector, and of three where marked, entries 0 / 1 / 2 / 3 in
+// complex64 and 4 / 5 / 6 / 24 in complex128 (rows x columns; the GPU steps such
+// times in units of 2):
+//    126 x 126  10.3 /  8.2 /  8.2 /  6.2    26.7 / 16.4 / 13.6 / 14.4
+//    364 x 91   10.3 /  8.2 /  8.2 / 10.0    36.9 / 14.4 / 20.5 / 14.4
+//    462 x 330  10.3 /  8.2 /  8.2 / 10.3    35.7 / 24.6 / 26.3 / 22.6
+//    792 x 66   20.5 / 20.5 / 18.5 / 28.7     152 / 47.3 / 71.6 / 51.6  (three)
+//    792 x 924  20.5 / 18.5 / 20.5 / 24.6     189 /  142 /  136 /  136
+//    924 x 220  12.3 / 14.4 / 12.3 / 16.4
+//    924 x 924  22.6 / 22.6 / 24.5 / 28.7     230 /  162 /  156 /  157
+//   1001 x 1001 22.6 / 24.8 / 24.4 / 32.8     208 /  150 /  145 /  145
+//   1287 x 715  22.6 / 20.5 / 23.5 / 26.6
+//   1820 x 560  30.8 / 24.6 / 31.8 / 36.9
+//   2002 x 364  20.5 / 20.5 / 18.9 / 28.7     159 /  109 /  113 /  105
+//   3432 x 91   28.7 / 26.6 / 22.6 / 41.0     194 / 70.4 /  103 / 73.7
+// (Entry 24 spills 92 bytes a thread at its 80 registers, entry 5 300 at 64.)
+int apply_small_config(bool fp64, int64_t rows, int max_dim_dn) {
   if (fp64) return rows <= 304 ? 6 : 24;
-  return rows <= 304 ? 3 : rows <= 912 ? 1 : 2;
+  if (rows <= 304) return 3;
+  if (max_dim_dn > 512) return rows > 912 && rows <= 1216 ? 0 : 1;
+  return rows <= 912 ? 1 : 2;
 }
 
 LaunchShape apply_shape(int max_dim_up, int max_dim_dn, bool fp64, int n_groups) {

@@ -127,8 +127,8 @@ int apply_config_count();
 bool apply_config_info(int i, int* fp64, int* nr, int* pp, int* minb, int* split, int* tma,
                        int* mv);
 // The configuration for small problems (where it is feasible; else the first
-// candidate), by the rows of all vectors together.
-int apply_small_config(bool fp64, int64_t rows);
+// candidate), by the rows of all vectors together and the longest row.
+int apply_small_config(bool fp64, int64_t rows, int max_dim_dn);
 // The default configuration (first candidate).
 LaunchShape apply_shape(int max_dim_up, int max_dim_dn, bool fp64, int n_groups);
 // Raise the dynamic shared-memory limit of the apply kernel for this shape
