@@ -311,11 +311,12 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   // largest-magnitude element real and positive
   CK(ctx, launch_permute_cols(true, yp, (int)ctx->dim_up, (int)ctx->dim_dn,
                               static_cast<const int32_t*>(ctx->sec.dn_order.p), false, s));
-  const bool to_device = is_device_ptr(psi);
-  double2* out = to_device ? static_cast<double2*>(psi) : wp;
+  // (written straight to a device psi that takes 16-byte stores, else copied)
+  const bool direct = is_device_ptr(psi) && ((uintptr_t)psi & 15u) == 0;
+  double2* out = direct ? static_cast<double2*>(psi) : wp;
   double* val = static_cast<double*>(phase.p);
   CK(ctx, launch_gs_phase(yp, out, D, val, reinterpret_cast<int64_t*>(val + kGsPhaseBlocks), s));
-  if (!to_device) CK(ctx, cudaMemcpyAsync(psi, wp, (size_t)D * 16, cudaMemcpyDeviceToHost, s));
+  if (!direct) CK(ctx, cudaMemcpyAsync(psi, wp, (size_t)D * 16, cudaMemcpyDefault, s));
   CK(ctx, cudaStreamSynchronize(s));
   *E0 = theta;
   if (resid_out) *resid_out = resid;
