@@ -213,14 +213,13 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
                 "not enough device memory (or workspace limit) for two Lanczos vectors");
   if (D == 1) K = 1;
   // V: K + 1 Lanczos vectors and the Ritz vector y
-  DevMem V, w, part, red, sdev, dots, coef, scal, phase;
+  DevMem V, w, part, red, sdev, coef, scal, phase;
   CK(ctx, V.alloc((size_t)(K + 2) * D * 16));
   CK(ctx, w.alloc((size_t)D * 16));
   const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(kGsMaxBlocks, (D + 2047) / 2048));
   CK(ctx, part.alloc(sizeof(double) * 2 * kGsMaxBlocks));
   CK(ctx, red.alloc(sizeof(double) * 2 + sizeof(unsigned)));
   CK(ctx, sdev.alloc(sizeof(double) * (K + 1)));
-  CK(ctx, dots.alloc(sizeof(double) * (size_t)gs_dot_blocks(D) * K));
   CK(ctx, coef.alloc(sizeof(double) * K));
   CK(ctx, scal.alloc(sizeof(GsScalars)));
   CK(ctx, phase.alloc(kGsPhaseBlocks * (sizeof(double) + sizeof(int64_t))));
@@ -250,9 +249,8 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   auto enqueue = [&](int k) -> cudaError_t {
     cudaError_t e = gs_apply(G, k, s);
     if (e == cudaSuccess)
-      e = launch_gs_step(Vp, D, k, wp, sc_dev, static_cast<double*>(dots.p),
-                         static_cast<double*>(coef.p), static_cast<double*>(part.p), counter,
-                         vk(k + 1), s);
+      e = launch_gs_step(Vp, D, k, wp, sc_dev, static_cast<double*>(coef.p),
+                         static_cast<double*>(part.p), counter, vk(k + 1), s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(H.p + 2 * k, sc_dev->alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess)

@@ -281,21 +281,26 @@ int grid_of(int64_t n, int per) {
 // large ones keep the partial sums small at Ns = 14 and 16
 bool wide(int64_t D) { return D > (int64_t)kGsMaxBlocks * 4 * kThreads; }
 
-}  // namespace
-
-int64_t gs_dot_blocks(int64_t D) {
+int64_t dot_blocks(int64_t D) {
   const int64_t per = (wide(D) ? 16 : 4) * (int64_t)kThreads;
   return (D + per - 1) / per;
 }
 
+}  // namespace
+
 cudaError_t launch_gs_step(const double2* V, int64_t D, int k, double2* w, GsScalars* S,
-                           double* dots, double* coef, double* partials, unsigned* counter,
-                           double2* vnext, cudaStream_t s) {
+                           double* coef, double* partials, unsigned* counter, double2* vnext,
+                           cudaStream_t s) {
+  // The partial projections, dot_blocks(D) x (k + 1) doubles, go where v_{k+1}
+  // will be: 2 D doubles, and k < D, k < kGsMaxVectors make them fit (one block
+  // up to 1024 elements, at most D / 1024 + 1 blocks of 200 above).
+  double* dots = reinterpret_cast<double*>(vnext);
   const int g = grid_of(D, 2 * kThreads);
   const double2* vk = V + (size_t)k * D;
   k_gs_dot<<<g, kThreads, 0, s>>>(vk, w, D, S, k, partials, counter);
   k_gs_sub<<<g, kThreads, 0, s>>>(w, vk, k > 0 ? vk - D : nullptr, D, S, k, partials, counter);
-  const int nb = (int)gs_dot_blocks(D), n = k + 1;
+  const int nb = (int)dot_blocks(D), n = k + 1;
+  if ((int64_t)nb * n > 2 * D) return cudaErrorInvalidValue;
   for (int pass = 0; pass < 2; ++pass) {
     if (wide(D)) k_gs_multidot<16><<<nb, kThreads, 0, s>>>(V, D, n, w, D, dots, S);
     else k_gs_multidot<4><<<nb, kThreads, 0, s>>>(V, D, n, w, D, dots, S);

@@ -232,15 +232,14 @@ struct GsScalars {
   double before, norm2;   // |w|^2 before the projections, and after
   int again;              // whether the next projection pass runs
 };
-// Blocks (rows of `dots`) of the projection kernel for vectors of D elements.
-int64_t gs_dot_blocks(int64_t D);
 // The rest of Lanczos step k after w = H v_k (ground.cu): alpha_k, the
 // three-term recursion, the projection against v_0 .. v_k (V: vectors of D
-// elements back to back), beta_k and vnext = v_{k+1}.  dots: gs_dot_blocks(D)
-// x (k + 1) doubles, coef: k + 1, partials: kGsMaxBlocks, counter: one zero.
+// elements back to back), beta_k and vnext = v_{k+1}, which holds the partial
+// projections until then.  coef: k + 1, partials: kGsMaxBlocks, counter: one
+// zero.
 cudaError_t launch_gs_step(const double2* V, int64_t D, int k, double2* w, GsScalars* S,
-                           double* dots, double* coef, double* partials, unsigned* counter,
-                           double2* vnext, cudaStream_t s);
+                           double* coef, double* partials, unsigned* counter, double2* vnext,
+                           cudaStream_t s);
 // out = y times the phase that makes its largest element (the first of the
 // largest) real and positive; val, idx: kGsPhaseBlocks entries of scratch.
 cudaError_t launch_gs_phase(const double2* y, double2* out, int64_t D, double* val, int64_t* idx,
