@@ -176,15 +176,17 @@ cudaError_t gs_apply(GsApply& G, int i, cudaStream_t s) {
   return launch_apply(true, a, G.nblk, G.shape, 0, s);
 }
 
-// Pinned host memory and events of a solve's pipeline.
-struct GsHost {
-  double* p = nullptr;   // [kGsMaxVectors][2]: alpha_k, beta_k
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  ~GsHost() {
-    if (p) cudaFreeHost(p);
-    for (cudaEvent_t e : ev)
-      if (e) cudaEventDestroy(e);
-  }
+// Small device arrays of a solve, one allocation (the addresses of its members
+// are taken on the host).
+struct GsScratch {
+  double partials[2 * kGsMaxBlocks];
+  double red[2];
+  double ritz[kGsMaxVectors + 1];
+  double coef[kGsMaxVectors];
+  double max_val[kGsPhaseBlocks];
+  int64_t max_idx[kGsPhaseBlocks];
+  GsScalars scal;
+  unsigned counter;
 };
 
 }  // namespace
@@ -213,33 +215,29 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
                 "not enough device memory (or workspace limit) for two Lanczos vectors");
   if (D == 1) K = 1;
   // V: K + 1 Lanczos vectors and the Ritz vector y
-  DevMem V, w, part, red, sdev, coef, scal, phase;
+  DevMem V, w, scratch;
   CK(ctx, V.alloc((size_t)(K + 2) * D * 16));
   CK(ctx, w.alloc((size_t)D * 16));
+  CK(ctx, scratch.alloc(sizeof(GsScratch)));
+  GsScratch* const g = static_cast<GsScratch*>(scratch.p);
   const int nblk = (int)std::max<int64_t>(1, std::min<int64_t>(kGsMaxBlocks, (D + 2047) / 2048));
-  CK(ctx, part.alloc(sizeof(double) * 2 * kGsMaxBlocks));
-  CK(ctx, red.alloc(sizeof(double) * 2 + sizeof(unsigned)));
-  CK(ctx, sdev.alloc(sizeof(double) * (K + 1)));
-  CK(ctx, coef.alloc(sizeof(double) * K));
-  CK(ctx, scal.alloc(sizeof(GsScalars)));
-  CK(ctx, phase.alloc(kGsPhaseBlocks * (sizeof(double) + sizeof(int64_t))));
   GsApply G;
   CKS(ctx, gs_apply_setup(G, ctx, static_cast<const double2*>(V.p), K + 2,
                          static_cast<double2*>(w.p), s));
   double2* Vp = static_cast<double2*>(V.p);
   double2* wp = static_cast<double2*>(w.p);
   double2* yp = Vp + (size_t)(K + 1) * D;
-  double* redp = static_cast<double*>(red.p);
-  unsigned* counter = reinterpret_cast<unsigned*>(redp + 2);
-  CK(ctx, cudaMemsetAsync(counter, 0, sizeof(unsigned), s));
-  GsScalars* sc_dev = static_cast<GsScalars*>(scal.p);
-  GsHost H;
-  CK(ctx, cudaHostAlloc(reinterpret_cast<void**>(&H.p), sizeof(double) * 2 * kGsMaxVectors,
-                        cudaHostAllocDefault));
-  for (cudaEvent_t& e : H.ev) CK(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  double* redp = g->red;
+  CK(ctx, cudaMemsetAsync(&g->counter, 0, sizeof(unsigned), s));
+  GsHost& H = ctx->gs_host;
+  if (!H.p)
+    CK(ctx, cudaHostAlloc(reinterpret_cast<void**>(&H.p), sizeof(double) * 2 * kGsMaxVectors,
+                          cudaHostAllocDefault));
+  for (cudaEvent_t& e : H.ev)
+    if (!e) CK(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   auto vk = [&](int k) { return Vp + (size_t)k * D; };
   auto norm_dot = [&](const double2* a, const double2* b, double out[2]) -> cudaError_t {
-    cudaError_t e = launch_norm_dot(a, b, D, static_cast<double*>(part.p), nblk, redp, s);
+    cudaError_t e = launch_norm_dot(a, b, D, g->partials, nblk, redp, s);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(out, redp, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e != cudaSuccess) return e;
@@ -249,12 +247,11 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   auto enqueue = [&](int k) -> cudaError_t {
     cudaError_t e = gs_apply(G, k, s);
     if (e == cudaSuccess)
-      e = launch_gs_step(Vp, D, k, wp, sc_dev, static_cast<double*>(coef.p),
-                         static_cast<double*>(part.p), counter, vk(k + 1), s);
+      e = launch_gs_step(Vp, D, k, wp, &g->scal, g->coef, g->partials, &g->counter, vk(k + 1), s);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(H.p + 2 * k, sc_dev->alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+      e = cudaMemcpyAsync(H.p + 2 * k, g->scal.alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(H.p + 2 * k + 1, sc_dev->beta + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+      e = cudaMemcpyAsync(H.p + 2 * k + 1, g->scal.beta + k, sizeof(double), cudaMemcpyDeviceToHost, s);
     return e == cudaSuccess ? cudaEventRecord(H.ev[k & 1], s) : e;
   };
   // seeded start vector, normalised
@@ -286,8 +283,8 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
       if (est <= 0.1 * tol * sc || b <= 1e-14 * sc || k + 1 == K || applies >= max_iter) break;
     }
     // Ritz vector y = V s, normalised
-    CK(ctx, cudaMemcpyAsync(sdev.p, sv.data(), sizeof(double) * sv.size(), cudaMemcpyHostToDevice, s));
-    CK(ctx, launch_combine_real(vk(0), D, (int)sv.size(), static_cast<double*>(sdev.p), yp, D, s));
+    CK(ctx, cudaMemcpyAsync(g->ritz, sv.data(), sizeof(double) * sv.size(), cudaMemcpyHostToDevice, s));
+    CK(ctx, launch_combine_real(vk(0), D, (int)sv.size(), g->ritz, yp, D, s));
     CK(ctx, norm_dot(yp, nullptr, nd));
     CK(ctx, cudaMemcpyAsync(redp, &nd[0], sizeof(double), cudaMemcpyHostToDevice, s));
     CK(ctx, launch_scale(yp, D, redp, true, s));
@@ -312,8 +309,7 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   // (written straight to a device psi that takes 16-byte stores, else copied)
   const bool direct = is_device_ptr(psi) && ((uintptr_t)psi & 15u) == 0;
   double2* out = direct ? static_cast<double2*>(psi) : wp;
-  double* val = static_cast<double*>(phase.p);
-  CK(ctx, launch_gs_phase(yp, out, D, val, reinterpret_cast<int64_t*>(val + kGsPhaseBlocks), s));
+  CK(ctx, launch_gs_phase(yp, out, D, g->max_val, g->max_idx, s));
   if (!direct) CK(ctx, cudaMemcpyAsync(psi, wp, (size_t)D * 16, cudaMemcpyDefault, s));
   CK(ctx, cudaStreamSynchronize(s));
   *E0 = theta;
