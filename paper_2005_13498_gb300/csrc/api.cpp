@@ -772,14 +772,7 @@ ed_status ed_double_occupation(ed_ctx* ctx, const void* psi, ed_dtype dtype, dou
   }
   if (!ctx->docc.p) CK(ctx, ctx->docc.alloc(kDoccScratchDoubles * sizeof(double)));
   double* scratch = static_cast<double*>(ctx->docc.p);
-  CK(ctx, launch_docc_sites(fp64, p, ctx->sec.dev, scratch, s));
-  double h[kDoccVals];
-  CK(ctx, cudaMemcpyAsync(h, scratch + kDoccScratchDoubles - kDoccVals, sizeof(h),
-                          cudaMemcpyDeviceToHost, s));
-  CK(ctx, cudaStreamSynchronize(s));
-  *d_avg = docc_average(h, ctx->Ns);
-  if (d_site)
-    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[i];
+  CK(ctx, docc_sites(fp64, p, ctx->sec.dev, ctx->Ns, scratch, d_avg, d_site, s));
   return ED_OK;
 }
 

@@ -1,5 +1,5 @@
 // Per-site double occupancies <n_i,up n_i,dn> = sum over u, d that both
-// contain site i of |psi_ud|^2 (Eq. (13)), shared by ed_double_occupation and
+// contain site i of |psi_ud|^2 (Eq. (13)), for ed_double_occupation and
 // ed_double_occupation_static.
 //
 // Bound by the FP64 pipe (two operations per cycle and SM), so the additions
@@ -189,6 +189,26 @@ k_docc_sum(const double* partial, int blocks, double* out) {
 // scratch: the partial sums, then kDoccVals results
 static_assert(kDoccScratchDoubles == (size_t)(kDoccBlocks + 1) * kDoccVals, "docc scratch");
 
+// partial[0][block] = sum of (sites in both u and d) |psi_ud|^2 over the block's
+// elements: the average where |psi|^2 is not finite, in which every element
+// counts, also one that no site weighs (0 times infinity is not a number).
+template <typename C>
+static __global__ void __launch_bounds__(kDoccThreads)
+k_docc_weighted(const C* psi, SectorDev sd, double* partial) {
+  __shared__ double red[kDoccThreads / 32];
+  const int64_t D = (int64_t)sd.dim_up * sd.dim_dn;
+  double v[1] = {0.0};
+  for (int64_t t = blockIdx.x * (int64_t)kDoccThreads + threadIdx.x; t < D;
+       t += (int64_t)gridDim.x * kDoccThreads) {
+    const int u = (int)(t / sd.dim_dn), d = (int)(t - (int64_t)u * sd.dim_dn);
+    const C p = psi[t];
+    const double q = (double)p.x * p.x + (double)p.y * p.y;
+    v[0] += __popc(__ldg(sd.up_word + u) & __ldg(sd.dn_word + d)) * q;
+  }
+  block_reduce<1>(v, red);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v[0];
+}
+
 static inline cudaError_t launch_docc(bool fp64, const void* psi, const SectorDev& sd, double* scratch,
                                       cudaStream_t s) {
   const DoccShape h = docc_shape(sd.dim_up, sd.dim_dn);
@@ -201,6 +221,21 @@ static inline cudaError_t launch_docc(bool fp64, const void* psi, const SectorDe
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_docc_sum<<<1, 32 * kDoccVals, 0, s>>>(scratch, h.blocks, scratch + (size_t)kDoccBlocks * kDoccVals);
+  return cudaGetLastError();
+}
+
+static inline cudaError_t launch_docc_weighted(bool fp64, const void* psi, const SectorDev& sd,
+                                               double* scratch, cudaStream_t s) {
+  const int64_t D = (int64_t)sd.dim_up * sd.dim_dn;
+  const int nb = (int)std::min<int64_t>(kDoccBlocks, (D + kDoccThreads - 1) / kDoccThreads);
+  if (fp64)
+    k_docc_weighted<<<nb, kDoccThreads, 0, s>>>(static_cast<const double2*>(psi), sd, scratch);
+  else
+    k_docc_weighted<<<nb, kDoccThreads, 0, s>>>(static_cast<const float2*>(psi), sd, scratch);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  // (the other sums of k_docc_sum are not read)
+  k_docc_sum<<<1, 32 * kDoccVals, 0, s>>>(scratch, nb, scratch + (size_t)kDoccBlocks * kDoccVals);
   return cudaGetLastError();
 }
 

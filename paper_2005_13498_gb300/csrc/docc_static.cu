@@ -10,7 +10,7 @@
 #include <mutex>
 
 #include "ctx.h"
-#include "docc.cuh"
+#include "kernels.cuh"
 
 namespace ed {
 
@@ -72,13 +72,6 @@ extern "C" ed_status ed_double_occupation_static(ed_ctx* ctx, const void* psi, e
   double* scratch = nullptr;
   CK(ctx, scratch_address(&scratch));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  CK(ctx, launch_docc(dtype == ED_C128, psi, ctx->sec.dev, scratch, s));
-  double h[kDoccVals];
-  CK(ctx, cudaMemcpyAsync(h, scratch + kDoccScratchDoubles - kDoccVals, sizeof(h),
-                          cudaMemcpyDeviceToHost, s));
-  CK(ctx, cudaStreamSynchronize(s));
-  *d_avg = docc_average(h, ctx->Ns);
-  if (d_site)
-    for (int i = 0; i < ctx->Ns; ++i) d_site[i] = h[i];
+  CK(ctx, docc_sites(dtype == ED_C128, psi, ctx->sec.dev, ctx->Ns, scratch, d_avg, d_site, s));
   return ED_OK;
 }

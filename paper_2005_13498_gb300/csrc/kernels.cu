@@ -21,6 +21,7 @@
 #include "device.cuh"
 #include "docc.cuh"
 
+#include <cmath>
 #include <cstdio>
 
 namespace ed {
@@ -2268,9 +2269,30 @@ cudaError_t launch_random_fill(double2* x, int64_t D, uint64_t seed, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_docc_sites(bool fp64, const void* psi, const SectorDev& sec, double* scratch,
-                              cudaStream_t s) {
-  return launch_docc(fp64, psi, sec, scratch, s);
+cudaError_t docc_sites(bool fp64, const void* psi, const SectorDev& sec, int Ns, double* scratch,
+                       double* d_avg, double* d_site, cudaStream_t s) {
+  double h[kDoccVals];   // the sites, then |psi|^2
+  auto fetch = [&]() -> cudaError_t {
+    const cudaError_t e = cudaMemcpyAsync(h, scratch + kDoccScratchDoubles - kDoccVals, sizeof(h),
+                                          cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess ? cudaStreamSynchronize(s) : e;
+  };
+  cudaError_t e = launch_docc(fp64, psi, sec, scratch, s);
+  if (e == cudaSuccess) e = fetch();
+  if (e != cudaSuccess) return e;
+  double sum = 0.0;
+  for (int i = 0; i < Ns; ++i) {
+    sum += h[i];
+    if (d_site) d_site[i] = h[i];
+  }
+  if (!std::isfinite(h[kMaxSites])) {
+    e = launch_docc_weighted(fp64, psi, sec, scratch, s);
+    if (e == cudaSuccess) e = fetch();
+    if (e != cudaSuccess) return e;
+    sum = h[0];
+  }
+  *d_avg = sum / Ns;
+  return cudaSuccess;
 }
 
 cudaError_t launch_convert(const void* in, bool in_fp64, void* out, bool out_fp64,

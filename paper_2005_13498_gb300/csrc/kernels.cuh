@@ -260,19 +260,13 @@ cudaError_t launch_axpy_real(double2* y, const double2* x, int64_t D,
                              cudaStream_t s);
 cudaError_t launch_random_fill(double2* x, int64_t D, uint64_t seed,
                                cudaStream_t s);
-// double occupancy: scratch (kDoccScratchDoubles) ends with kDoccVals sums,
-// the kMaxSites per-site values and |psi|^2
+// Double occupancies of psi (device): the average over the sites and, unless
+// d_site is null, the value of each of the Ns sites.  scratch holds
+// kDoccScratchDoubles on the device.  Synchronises s.
 constexpr int kDoccVals = kMaxSites + 1;
 constexpr size_t kDoccScratchDoubles = (size_t)(1024 + 1) * kDoccVals;
-// The average from the sums h: 0 |psi|^2 is 0 unless an element of psi is
-// not finite, which must show in the average wherever it stands.
-inline double docc_average(const double* h, int Ns) {
-  double s = 0.0 * h[kMaxSites];
-  for (int i = 0; i < Ns; ++i) s += h[i];
-  return s / Ns;
-}
-cudaError_t launch_docc_sites(bool fp64, const void* psi, const SectorDev& sec, double* scratch,
-                              cudaStream_t s);
+cudaError_t docc_sites(bool fp64, const void* psi, const SectorDev& sec, int Ns, double* scratch,
+                       double* d_avg, double* d_site, cudaStream_t s);
 // dtype conversion
 cudaError_t launch_convert(const void* in, bool in_fp64, void* out,
                            bool out_fp64, int64_t n_complex, cudaStream_t s);
