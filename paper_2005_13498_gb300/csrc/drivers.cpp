@@ -176,6 +176,13 @@ cudaError_t gs_apply(GsApply& G, int i, cudaStream_t s) {
   return launch_apply(true, a, G.nblk, G.shape, 0, s);
 }
 
+// Vectors up to which a solve waits for each step instead of enqueuing the next
+// one ahead: the pinned memory that takes costs a context 0.25 ms once.  us of a
+// context's only solve and its end, waiting / ahead: 3 states 801 / 1062, 4
+// states 933 / 1172, 16 states 1865 / 1969, 25 states 2712 / 2685; of a later
+// solve 475 / 437, 550 / 492, 1476 / 1321, 2356 / 2024.
+constexpr int kGsAhead = 4;
+
 // Small device arrays of a solve, one allocation (the addresses of its members
 // are taken on the host).
 struct GsScratch {
@@ -229,12 +236,18 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   double2* yp = Vp + (size_t)(K + 1) * D;
   double* redp = g->red;
   CK(ctx, cudaMemsetAsync(&g->counter, 0, sizeof(unsigned), s));
+  // alpha_k and beta_k on the host; with more than kGsAhead vectors step k + 1
+  // is on the stream while the host examines step k, which takes pinned memory
+  const bool ahead = K > kGsAhead;
+  double pageable[2 * kGsAhead];
   GsHost& H = ctx->gs_host;
-  if (!H.p)
+  if (ahead && !H.p)
     CK(ctx, cudaHostAlloc(reinterpret_cast<void**>(&H.p), sizeof(double) * 2 * kGsMaxVectors,
                           cudaHostAllocDefault));
-  for (cudaEvent_t& e : H.ev)
-    if (!e) CK(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  if (ahead)
+    for (cudaEvent_t& e : H.ev)
+      if (!e) CK(ctx, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  double* const ab = ahead ? H.p : pageable;
   auto vk = [&](int k) { return Vp + (size_t)k * D; };
   auto norm_dot = [&](const double2* a, const double2* b, double out[2]) -> cudaError_t {
     cudaError_t e = launch_norm_dot(a, b, D, g->partials, nblk, redp, s);
@@ -249,10 +262,10 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
     if (e == cudaSuccess)
       e = launch_gs_step(Vp, D, k, wp, &g->scal, g->coef, g->partials, &g->counter, vk(k + 1), s);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(H.p + 2 * k, g->scal.alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+      e = cudaMemcpyAsync(ab + 2 * k, g->scal.alpha + k, sizeof(double), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess)
-      e = cudaMemcpyAsync(H.p + 2 * k + 1, g->scal.beta + k, sizeof(double), cudaMemcpyDeviceToHost, s);
-    return e == cudaSuccess ? cudaEventRecord(H.ev[k & 1], s) : e;
+      e = cudaMemcpyAsync(ab + 2 * k + 1, g->scal.beta + k, sizeof(double), cudaMemcpyDeviceToHost, s);
+    return e == cudaSuccess && ahead ? cudaEventRecord(H.ev[k & 1], s) : e;
   };
   // seeded start vector, normalised
   CK(ctx, launch_random_fill(vk(0), D, seed, s));
@@ -267,15 +280,15 @@ ed_status ed_ground_state(ed_ctx* ctx, void* psi, double* E0, double tol, int ma
   while (applies < max_iter && !converged) {
     al.clear();
     be.clear();
-    // step k + 1 is on the stream while the host examines step k; when step
-    // k turns out to be the last, the work of step k + 1 is discarded
-    CK(ctx, enqueue(0));
+    // (when step k turns out to be the last, a step k + 1 is discarded)
+    if (ahead) CK(ctx, enqueue(0));
     for (int k = 0; k < K; ++k) {
-      if (k + 1 < K) CK(ctx, enqueue(k + 1));
-      CK(ctx, cudaEventSynchronize(H.ev[k & 1]));
+      const int next = ahead ? k + 1 : k;
+      if (next < K) CK(ctx, enqueue(next));
+      CK(ctx, ahead ? cudaEventSynchronize(H.ev[k & 1]) : cudaStreamSynchronize(s));
       ++applies;
-      al.push_back(H.p[2 * k]);
-      const double b = H.p[2 * k + 1];
+      al.push_back(ab[2 * k]);
+      const double b = ab[2 * k + 1];
       be.push_back(b);
       lowest_eigenpair(al, be, &theta, sv);
       const double est = b * std::fabs(sv.back());

@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("lat,nu,nd", [(synth.ring(6), 3, 3), (synth.chain(3), 0, 2),
-                                       (synth.chain(2), 0, 0)])
+                                       (synth.chain(2), 0, 0),
+                                       (synth.dimer(), 1, 1), (synth.chain(5), 1, 0)])
 def test_result_buffers(ed_lib, lat, nu, nd):
     torch = torch_cuda()
     ed = ed_lib
