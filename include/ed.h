@@ -380,9 +380,9 @@ ed_status ed_apply_config_info(int config, int* fp64, int* rows_per_cta,
  * ed_apply_H plan and ground-state solve set up after the call (contexts
  * rebuild their plans when it changes).  config = -1 (the default): an
  * autotuner times the feasible entries once per precision and sector shape
- * (sectors under 2^20 elements take an entry by their number of rows, and
- * in complex64 ed_propagate runs sectors that fit the chip's shared memory in
- * a kernel of its own that has no entry); otherwise the
+ * (sectors under 2^20 elements take an entry by the number and the length of
+ * their rows, and in complex64 ed_propagate runs sectors that fit the chip's
+ * shared memory in a kernel of its own that has no entry); otherwise the
  * given entry is used, and calls whose precision or sector it does not fit
  * fail with ED_ERR_CUDA and a message naming it.  ED_ERR_ARG if config is
  * not -1 and not a table index.                                             */

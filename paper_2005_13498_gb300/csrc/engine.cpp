@@ -524,24 +524,26 @@ std::string Engine::begin(const std::vector<double>& coefs, const std::vector<do
   return "";
 }
 
-// Passes of the step graph that always run in the adaptive mode; with at least
-// kGateMinM vectors the others are the body of a conditional node.  Returning
-// at once, each of them costs its launches, and one more is computed and thrown
-// away where the exit is at kGatePass.  A step that needs the body waits for
-// the check of pass kGatePass, starts a graph within the graph, and launches
-// every pass from there a little later.  us per step, all passes launched /
-// the rest conditional, the first exit at most 9, the second at 11 to 13:
+// Passes of the step graph that always run in the adaptive mode; the others are
+// the body of a conditional node.  Returning at once, each of them costs its
+// launches, and one more is computed and thrown away where the exit is at
+// kGatePass.  A step that needs the body waits for the check of pass kGatePass,
+// starts a graph within the graph, and launches every pass from there a little
+// later.  us per step, all passes launched / the rest conditional, the first
+// exit at most 9, the second at 11 to 13:
 //                            m = 14                     m = 20                     m = 30
 //   8-site ring, c64      166/168    264/294      180/162    274/300      221/171    320/349
 //   10-site chain, c64    193/195    295/327      215/191    321/353      250/193    352/384
 //   12-site torus, c64    454/444    592/627      462/414    640/678      560/444    697/733
 //   the same, c128       1849/1837  2361/2401    1897/1843  2408/2448    1969/1839  2483/2522
 //   14-site ladder, c64  2346/2319  3290/3332    2181/2089  3364/3410    2538/2324  3479/3522
-// (and 2816/2588, 2890/2595 and 3002/2592 for the ladder's exit at 10).  What an
-// early exit gains grows with m, what a late one pays does not: the line is
-// where the two are alike for sectors between the chain and the torus.
+// (and 2816/2588, 2890/2595 and 3002/2592 for the ladder's exit at 10; at m = 16
+// the ring's early exits read 145/142, the chain's 176/166).  A maximum is chosen
+// well above the usual exit, so the line lies where an early exit begins to gain:
+// at 13 vectors, and at 15 for sectors under 2^18 elements, where the launches
+// of the three or four passes that 13 or 14 leave cost no more than the node.
 constexpr int kGatePass = 10;
-constexpr int kGateMinM = 20;
+static int gate_min_m(int64_t elements) { return elements < ((int64_t)1 << 18) ? 15 : 13; }
 
 namespace {
 // Records around a launch in profile mode, then the launch.
@@ -598,7 +600,9 @@ std::string Engine::launch_step(cudaStream_t s, bool profile, cudaEvent_t* ev, i
   const bool f = cfg_.fp64;
   Marks mk{profile, ev, kind_of, nev};
   std::string err;
-  const bool gated = cfg_.eps_tol > 0.0 && !profile && cfg_.m >= kGateMinM;
+  int64_t elements = 0;
+  for (const EngineVector& v : vecs_) elements += v.D;
+  const bool gated = cfg_.eps_tol > 0.0 && !profile && cfg_.m >= gate_min_m(elements);
   err = launch_passes(s, side_, 1, gated ? kGatePass : cfg_.m, profile, ev, kind_of, nev);
   if (!err.empty()) return err;
   if (gated) {   // s is being captured (capture())
