@@ -428,16 +428,22 @@ std::string Engine::setup_persistent(const SpinTable* up, bool vec_ok) {
   kry_deg_ = 1;
   for (int r = 0; r < up->dim; ++r) kry_deg_ = std::max(kry_deg_, up->off[r + 1] - up->off[r]);
   kry_vec_ = vec_ok;
+  auto smem_of = [&](int steps) {
+    return krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_,
+                       krylov_coef_rows(steps, cfg_.energy));
+  };
   // as many sub-steps per launch as their coefficients leave room for
   int ctas = 0;
   for (kry_steps_ = kKrylovSteps; kry_steps_ > 0; --kry_steps_) {
-    kry_smem_ = krylov_smem(kry_rows_, sd.dim_dn, kry_deg_, n_groups_,
-                            krylov_coef_rows(kry_steps_, cfg_.energy));
-    if (kry_smem_ > 227 * 1024) continue;
-    ED_TRY(krylov_prepare(kry_vec_, kry_smem_, &ctas));
+    if (smem_of(kry_steps_) > 227 * 1024) continue;
+    ED_TRY(krylov_prepare(kry_vec_, smem_of(kry_steps_), &ctas));
     if (ctas > 0) break;
   }
   if (ctas < 1) return "";
+  // and fewer, down to half, if that leaves the gathers a larger L1 cache
+  for (int n = kry_steps_; 2 * n >= kKrylovSteps; --n)
+    if (krylov_carveout(smem_of(n)) < krylov_carveout(smem_of(kry_steps_))) kry_steps_ = n;
+  kry_smem_ = smem_of(kry_steps_);
   ED_TRY(d_slots_.alloc(kKrylovSlotBytes));
   kry_grid_ = grid;
   return "";

@@ -218,6 +218,9 @@ __host__ __device__ constexpr int krylov_coef_rows(int n_steps, int energy) {
 // Dynamic shared memory of a launch, and the CTAs per SM it allows (0: does
 // not fit); krylov_prepare raises the kernel's limit.
 size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows);
+// KiB of the SM's memory that a launch takes from its L1 cache: the sizes shared
+// memory can have there, the block's static arrays and the system's 1 KiB counted.
+int krylov_carveout(size_t smem);
 cudaError_t krylov_prepare(bool vec, size_t smem, int* ctas_per_sm);
 cudaError_t launch_krylov(bool vec, const KrylovArgs& k, int grid, size_t smem,
                           cudaStream_t s);

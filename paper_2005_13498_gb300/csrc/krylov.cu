@@ -59,8 +59,9 @@ using TIO = TileIO<float2, NR>;
 // Scalars of the Lanczos recursion in shared memory, 1-based as LanczosState.
 struct Scalars {
   double alpha[kMaxKrylov + 2], beta[kMaxKrylov + 2], inv[kMaxKrylov + 2];
-  double al[64], be[64], yre[64], yim[64], pre[64], pim[64];
-  double yprev_re[kMaxKrylov], yprev_im[kMaxKrylov];
+  double al[64], be[64], yre[64], yim[64];
+  // y of the check before, or of one vector less in the step's exponential
+  double yprev_re[64], yprev_im[64];
   double tot[2], part[2][4];
   double beta0, scale, as, conv_delta;
   double utab[kMaxSites + 1];   // U n
@@ -214,7 +215,7 @@ __device__ __forceinline__ void ldcg_pair(const float2* row, int p, int dim, flo
 template <bool VEC>
 __device__ __forceinline__ void off_diagonal(
     const SectorDev& sd, const float2* tile, int t, int pcl, const float2* x,
-    const uint2* const (&list)[NR], const int (&deg)[NR], const float2* coefQ,
+    const uint2* const (&list)[NR], const int (&deg)[NR], const float2* coefQ, const float2* coefS,
     float2 (&acc)[NR][2]) {
   const int lane = threadIdx.x & 31;
   const int dim_dn = sd.dim_dn;
@@ -228,7 +229,7 @@ __device__ __forceinline__ void off_diagonal(
     acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
   }
   auto flush = [&](uint32_t g) {
-    const float2 c = coefQ[1 + 2 * g];
+    const float2 c = coefS[g];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       cmac(acc[r][0], c, s0[r]);
@@ -349,7 +350,7 @@ struct Share {
   SectorDev sd;
   VecDev vd;
   int off_w, off_q, off_l, off_d;   // byte offsets of the arrays below
-  int n_coef, max_deg, nloc, ld, npairs, ntile, items, nwork;
+  int n_groups, max_deg, nloc, ld, npairs, ntile, items, nwork;
 };
 constexpr int kOffShare = (sizeof(Scalars) + 15) & ~15;
 constexpr int kOffX = (kOffShare + sizeof(Share) + 15) & ~15;
@@ -358,13 +359,13 @@ __device__ __forceinline__ Share& share() { return *reinterpret_cast<Share*>(sme
 // rows of x_j and w: [tile rows][dim_dn + zero columns][NR]
 __device__ __forceinline__ float2* tile_x() { return reinterpret_cast<float2*>(smem_raw + kOffX); }
 __device__ __forceinline__ float2* tile_w() { return reinterpret_cast<float2*>(smem_raw + share().off_w); }
-// Signed coefficients, 1 + 2 n_groups to a row (0, then c_g and -c_g of every
-// group): a row for each sub-step of the launch, then, with energies, one for
+// Coefficients, 3 n_groups to a row (c_g and -c_g of every group for T_up, then
+// c_g of every group for T_dn: 0.1 to 0.6 % faster than one table for both): a row for each sub-step of the launch, then, with energies, one for
 // its first time and one for the time after each sub-step.  All of them are
 // written before the first grid-wide sum and only read after it, so that no
 // pass depends on a hand-over within the launch.
 __device__ __forceinline__ const float2* coef_q(int row) {
-  return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * share().n_coef;
+  return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * 3 * share().n_groups;
 }
 // T_up entries [rows][max_deg]: source offset, coefficient slot; their numbers
 __device__ __forceinline__ uint2* up_list() { return reinterpret_cast<uint2*>(smem_raw + share().off_l); }
@@ -408,7 +409,7 @@ __device__ __forceinline__ double apply_pass(const float2* x, const float2* xp, 
       urow[r] = cta + (have ? li : 0) * G;
     }
     float2 acc[NR][2];
-    off_diagonal<VEC>(sd, tile, t, min(p, npairs - 1), x, lst, deg, coefQ, acc);
+    off_diagonal<VEC>(sd, tile, t, min(p, npairs - 1), x, lst, deg, coefQ, coefQ + 2 * h.n_groups, acc);
     if (p >= npairs) continue;
     const int d0 = 2 * p;
     const bool has1 = d0 + 1 < dim_dn;
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
   const int RB = (k.rows + NR - 1) / NR;
   const int tile_bytes = RB * ld * 16;
   const int off_q = kOffX + 2 * tile_bytes;
-  const int n_coef = 1 + 2 * a.n_groups;
+  const int n_coef = 3 * a.n_groups;   // to a row
   const int off_l = off_q + krylov_coef_rows(k.n_steps, k.energy) * n_coef * (int)sizeof(float2);
   float2* const tileX = tile_x();
   float2* const tileW = reinterpret_cast<float2*>(smem_raw + kOffX + tile_bytes);
@@ -508,7 +509,7 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
       const uint32_t en = __ldg(sd.up_ent + e0 + i);
       const uint32_t g = (en >> kEntGroupShift) & 0xFFu;
       list[(size_t)li * k.max_deg + i] =
-          make_uint2((en & kEntRankMask) * (uint32_t)dim_dn, 1u + 2u * g + (en >> 31));
+          make_uint2((en & kEntRankMask) * (uint32_t)dim_dn, 2u * g + (en >> 31));
     }
     if (tid == 0) degS[li] = ne;
   }
@@ -529,7 +530,7 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
   if (tid == 0) {
     h.off_w = kOffX + tile_bytes;
     h.off_q = off_q;
-    h.n_coef = n_coef;
+    h.n_groups = a.n_groups;
     h.off_l = off_l;
     h.off_d = off_l + k.rows * k.max_deg * (int)sizeof(uint2);
     h.max_deg = k.max_deg;
@@ -550,16 +551,13 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
 
   for (int i = tid; i < krylov_coef_rows(k.n_steps, k.energy) * n_coef; i += NT) {
     const int row = i / n_coef, slot = i - row * n_coef;
-    float2 q = make_float2(0.f, 0.f);
-    if (slot > 0) {
-      const bool obs = row >= k.n_steps;
-      const float2 c = reinterpret_cast<const float2*>(
-          obs ? a.coefs_obs : a.coefs)[(size_t)(step0 + row - (obs ? k.n_steps : 0)) * a.n_groups +
-                                       ((slot - 1) >> 1)];
-      const float sg = ((slot - 1) & 1) ? -1.f : 1.f;
-      q = make_float2(sg * c.x, sg * c.y);
-    }
-    coefQ[i] = q;
+    const int plain = slot - 2 * a.n_groups;   // T_dn's part from 0 on
+    const bool obs = row >= k.n_steps;
+    const float2 c = reinterpret_cast<const float2*>(
+        obs ? a.coefs_obs : a.coefs)[(size_t)(step0 + row - (obs ? k.n_steps : 0)) * a.n_groups +
+                                     (plain >= 0 ? plain : slot >> 1)];
+    const float sg = plain < 0 && (slot & 1) ? -1.f : 1.f;
+    coefQ[i] = make_float2(sg * c.x, sg * c.y);
   }
   block_sync();
   // one pass over the items: f(tile row, column tile, column pair)
@@ -737,13 +735,13 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
       block_sync();
       if (warp == 0) tridiag_expm_e1(S.al, S.be, n, a.tau, S.yre, S.yim);
       else if (warp == 1 && n > 1)
-        tridiag_expm_e1(S.al, S.be, n - 1, a.tau, S.pre, S.pim);
+        tridiag_expm_e1(S.al, S.be, n - 1, a.tau, S.yprev_re, S.yprev_im);
       block_sync();
       if (warp == 1) {
         double dn = 0.0, yn = 0.0;
         if (n > 1)
           for (int i = lane; i < n; i += 32) {
-            const double pr = i < n - 1 ? S.pre[i] : 0.0, pi = i < n - 1 ? S.pim[i] : 0.0;
+            const double pr = i < n - 1 ? S.yprev_re[i] : 0.0, pi = i < n - 1 ? S.yprev_im[i] : 0.0;
             dn += (S.yre[i] - pr) * (S.yre[i] - pr) + (S.yim[i] - pi) * (S.yim[i] - pi);
             yn += S.yre[i] * S.yre[i] + S.yim[i] * S.yim[i];
           }
@@ -825,7 +823,15 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
 size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows) {
   const size_t rb = (rows + NR - 1) / NR;
   return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 +
-         (size_t)coef_rows * (1 + 2 * n_groups) * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+         (size_t)coef_rows * 3 * n_groups * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+}
+
+int krylov_carveout(size_t smem) {
+  constexpr int kKiB[] = {8, 16, 32, 64, 100, 132, 164, 196, 228};
+  constexpr size_t own = NT * sizeof(double) + (kMaxKrylov + 2) * sizeof(float2) + 1024;
+  for (int c : kKiB)
+    if (smem + own <= (size_t)c * 1024) return c;
+  return 228;
 }
 
 template <bool VEC>

@@ -150,7 +150,8 @@ def test_rows_with_many_entries(ed_lib, rep):
 
 def test_room_for_few_steps(ed_lib):
     """182 bond groups and seven rows of 1001 columns in a CTA: with energies
-    the shared memory holds the coefficients of 14 steps, not of 16."""
+    the shared memory does not hold the coefficients of 16 steps, and a launch
+    is given fewer."""
     torch = torch_cuda()
     ed = ed_lib
     h = ed.Hubbard(synth.complete_graph(14, seed=1), 4, 4, 6.0)
