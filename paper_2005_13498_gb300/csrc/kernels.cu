@@ -1490,7 +1490,9 @@ __global__ void __launch_bounds__(256, 4) k_combine(BatchArgs a) {
   const VecDev vd = a.vec[eb.vec];
   LanczosState* st = a.st + eb.vec;
   const SectorDev sd = a.sec[vd.sector];
-  const int n = COMBINE ? st->m_eff : 1;
+  // a state of norm zero has no Krylov vectors: no pass has written the others
+  const bool vectors = COMBINE && st->beta0 > 0.0 && isfinite(st->beta0);
+  const int n = vectors ? st->m_eff : 1;
   if (COMBINE) {
     for (int jj = threadIdx.x; jj < n; jj += blockDim.x) {
       cf[jj].x = (R)st->comb_re[jj + 1];
