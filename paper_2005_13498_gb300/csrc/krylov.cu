@@ -755,7 +755,8 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
     }
     if (warp == 0)
       for (int i = lane; i < n; i += 32) {
-        const double f = zero ? 0.0 : S.beta0 * S.inv[i + 1];
+        // (a norm that is not finite goes on into the state, as in k_expm)
+        const double f = S.beta0 * S.inv[i + 1];
         const double re = f * S.yre[i], im = f * S.yim[i];
         cf[i].x = (float)re;
         cf[i].y = (float)im;

@@ -1,5 +1,6 @@
 """States of norm zero, alone and in a batch, on device memory that held
-not-a-number before: no vector that no pass has written may enter a result."""
+not-a-number before: no vector that no pass has written may enter a result.
+And the other end: a norm that is not finite."""
 import numpy as np
 import pytest
 
@@ -87,3 +88,24 @@ def test_batch_with_zero_vectors(ed_lib, dtype):
                 if not lives:      # c annihilates psi(0), not psi(t): the bra alone is not zero
                     assert np.abs(G[:, site, spin]).max() == 0.0
 
+
+
+@pytest.mark.parametrize("config", [-1, "pinned"])
+@pytest.mark.parametrize("lat,nu,nd", [(synth.ring(6), 3, 2), (synth.chain(5), 0, 2)])
+def test_norm_that_overflows(ed_lib, lat, nu, nd, config):
+    """complex64 elements whose squares are infinite: the call fails, and the
+    state it leaves shows it."""
+    torch = torch_cuda()
+    ed = ed_lib
+    h = ed.Hubbard(lat, nu, nd, 4.0)
+    x = to_dev(torch, 1e22 * synth.complex_normal(h.D, 3), "c64")
+    try:
+        ed.ed_set_apply_config(PINNED["c64"] if config == "pinned" else -1)
+        with pytest.raises(ed.EDError) as e:
+            ed.ed_propagate(h.ctx, x, ed.ED_C64, PULSE, 0.0, 0.02, 3, 12)
+        torch.cuda.synchronize()
+    finally:
+        ed.ed_set_apply_config(-1)
+        h.close()
+    assert e.value.status == 7
+    assert np.isnan(from_dev(x)).all()
