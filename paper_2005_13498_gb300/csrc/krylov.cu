@@ -216,7 +216,7 @@ __device__ __forceinline__ void ldcg_pair(const float2* row, int p, int dim, flo
 template <bool VEC>
 __device__ __forceinline__ void off_diagonal(
     const SectorDev& sd, const float2* tile, int t, int pcl, const float2* x,
-    const uint2* const (&list)[NR], const int (&deg)[NR], const float2* coefQ, const float2* coefS,
+    const uint2* const (&list)[NR], const int (&deg)[NR], const float2* coefQ,
     float2 (&acc)[NR][2]) {
   const int lane = threadIdx.x & 31;
   const int dim_dn = sd.dim_dn;
@@ -230,7 +230,7 @@ __device__ __forceinline__ void off_diagonal(
     acc[r][0] = acc[r][1] = make_float2(0.f, 0.f);
   }
   auto flush = [&](uint32_t g) {
-    const float2 c = coefS[g];
+    const float2 c = coefQ[2 * g];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
       cmac(acc[r][0], c, s0[r]);
@@ -360,13 +360,12 @@ __device__ __forceinline__ Share& share() { return *reinterpret_cast<Share*>(sme
 // rows of x_j and w: [tile rows][dim_dn + zero columns][NR]
 __device__ __forceinline__ float2* tile_x() { return reinterpret_cast<float2*>(smem_raw + kOffX); }
 __device__ __forceinline__ float2* tile_w() { return reinterpret_cast<float2*>(smem_raw + share().off_w); }
-// Coefficients, 3 n_groups to a row (c_g and -c_g of every group for T_up, then
-// c_g of every group for T_dn: 0.1 to 0.6 % faster than one table for both): a row for each sub-step of the launch, then, with energies, one for
+// Signed coefficients, 2 n_groups to a row (c_g and -c_g of every group): a row for each sub-step of the launch, then, with energies, one for
 // its first time and one for the time after each sub-step.  All of them are
 // written before the first grid-wide sum and only read after it, so that no
 // pass depends on a hand-over within the launch.
 __device__ __forceinline__ const float2* coef_q(int row) {
-  return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * 3 * share().n_groups;
+  return reinterpret_cast<const float2*>(smem_raw + share().off_q) + row * 2 * share().n_groups;
 }
 // T_up entries [rows][max_deg]: source offset, coefficient slot; their numbers
 __device__ __forceinline__ uint2* up_list() { return reinterpret_cast<uint2*>(smem_raw + share().off_l); }
@@ -410,7 +409,7 @@ __device__ __forceinline__ double apply_pass(const float2* x, const float2* xp, 
       urow[r] = cta + (have ? li : 0) * G;
     }
     float2 acc[NR][2];
-    off_diagonal<VEC>(sd, tile, t, min(p, npairs - 1), x, lst, deg, coefQ, coefQ + 2 * h.n_groups, acc);
+    off_diagonal<VEC>(sd, tile, t, min(p, npairs - 1), x, lst, deg, coefQ, acc);
     if (p >= npairs) continue;
     const int d0 = 2 * p;
     const bool has1 = d0 + 1 < dim_dn;
@@ -487,7 +486,7 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
   const int RB = (k.rows + NR - 1) / NR;
   const int tile_bytes = RB * ld * 16;
   const int off_q = kOffX + 2 * tile_bytes;
-  const int n_coef = 3 * a.n_groups;   // to a row
+  const int n_coef = 2 * a.n_groups;   // to a row
   const int off_l = off_q + krylov_coef_rows(k.n_steps, k.energy) * n_coef * (int)sizeof(float2);
   float2* const tileX = tile_x();
   float2* const tileW = reinterpret_cast<float2*>(smem_raw + kOffX + tile_bytes);
@@ -552,12 +551,11 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
 
   for (int i = tid; i < krylov_coef_rows(k.n_steps, k.energy) * n_coef; i += NT) {
     const int row = i / n_coef, slot = i - row * n_coef;
-    const int plain = slot - 2 * a.n_groups;   // T_dn's part from 0 on
     const bool obs = row >= k.n_steps;
     const float2 c = reinterpret_cast<const float2*>(
         obs ? a.coefs_obs : a.coefs)[(size_t)(step0 + row - (obs ? k.n_steps : 0)) * a.n_groups +
-                                     (plain >= 0 ? plain : slot >> 1)];
-    const float sg = plain < 0 && (slot & 1) ? -1.f : 1.f;
+                                     (slot >> 1)];
+    const float sg = (slot & 1) ? -1.f : 1.f;
     coefQ[i] = make_float2(sg * c.x, sg * c.y);
   }
   block_sync();
@@ -825,7 +823,7 @@ __global__ void __launch_bounds__(NT, 1) k_krylov(KrylovArgs k) {
 size_t krylov_smem(int rows, int dim_dn, int max_deg, int n_groups, int coef_rows) {
   const size_t rb = (rows + NR - 1) / NR;
   return kOffX + 2 * rb * (size_t)(dim_dn + kZeroCols) * 16 +
-         (size_t)coef_rows * 3 * n_groups * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
+         (size_t)coef_rows * 2 * n_groups * 8 + (size_t)rows * max_deg * 8 + (size_t)rows * 4;
 }
 
 int krylov_carveout(size_t smem) {
